@@ -52,13 +52,16 @@ int cuda_fail(cudaError_t e, const char *what, const char *file, int line) {
 
 template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
-                      cudaStream_t s, int shape, const T *geo, const T *rho, const GridBarrier *det) {
+                      cudaStream_t s, int shape, const T *geo, const T *geox, const T *rho, const GridBarrier *det) {
   if (shape == 5 || det) {
     // cell-component kernel (Laplacian form, constant rho); the column kernel serves the rest.
     // det: its deterministic cooperative form (setup admits deterministic mode only where it serves
     // every application of the solve)
     const bool generic_a = (mode & kApplyA) && ((mode & kApplySym) || rho);
     if (!generic_a) {
+      if constexpr (sizeof(T) == 8) {
+        if (!det && launch_cell_apply_fx(L, mode, u, p, yu, yp, geox, nullptr, s) == 0) return 0;
+      }
       const int r = L.k == 2 ? launch_cell_apply_cc_k<2, T>(L, mode, u, p, yu, yp, geo, det, s)
                              : (L.k == 3 ? launch_cell_apply_cc_k<3, T>(L, mode, u, p, yu, yp, geo, det, s) : -1);
       if (r == 0) return 0;
@@ -179,6 +182,7 @@ struct LevelRT {
   bool fuse = true;  // fused smoothing on this level (set by the setup's timing, when eligible)
   const T *geo = nullptr;  // 3D trilinear: precomputed per-point geometry the column kernel reads
   const T *geo_stored = nullptr;  // FP32: the stored geometry, used (geo) where the setup's timing keeps it
+  const T *geox = nullptr; // FP64, k = 2, trilinear: the fixed-point form's digits of it
   const T *rho = nullptr;  // per-cell density of the gamma rho mass term (null: rho = 1)
   const T *Ce = nullptr;   // packed element matrices of the stabilisation block C (null: on the fly)
   T *DAinv = nullptr, *DSinv = nullptr;
@@ -433,7 +437,7 @@ struct Runner {
       o.items = pq_items(o);
       return;
     }
-    launch_cell_apply<T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].shape, L[l].geo, L[l].rho,
+    launch_cell_apply<T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].shape, L[l].geo, L[l].geox, L[l].rho,
                          C->det ? &C->gb : nullptr);
     note();
   }
@@ -657,7 +661,11 @@ struct Runner {
   }
   void fapply(int l, int mode, const T *u, const T *p, T *yu, T *yp, const Fuse<T> &F) {
     if (L[l].shape == 5) {  // the cell-component kernel's fused form where it has one (k = 2)
-      const int r = launch_cell_apply_cc_fused_k<2, T>(L[l].d, mode, u, p, yu, yp, L[l].geo, F, s);
+      int r;
+      if constexpr (sizeof(T) == 8)
+        r = launch_cell_apply_fx(L[l].d, mode, u, p, yu, yp, L[l].geox, &F, s);
+      else
+        r = launch_cell_apply_cc_fused_k<2, T>(L[l].d, mode, u, p, yu, yp, L[l].geo, F, s);
       if (r == 0) {
         note();
         return;
@@ -1314,7 +1322,7 @@ template <typename T>
 static int autotune_level(stokes_ctx *C, LevelRT<T> &R, const Tab1D<T> *tab) {
   if (R.d.dim != 3) return STOKES_OK;
   const bool cc = cc_level_supported(R.d.dim, R.d.k, R.d.cartesian, sizeof(T)) && !C->sym && !R.rho &&
-                  (R.d.cartesian || sizeof(T) == 4 || R.geo);
+                  (R.d.cartesian || sizeof(T) == 4 || R.geox);
   const bool sg = R.geo_stored && !R.geo;
   // candidates: column shapes 4, 1, 3 (on-the-fly geometry), point kernel, cell-component kernel,
   // then the column shapes reading the stored geometry
@@ -1340,7 +1348,7 @@ static int autotune_level(stokes_ctx *C, LevelRT<T> &R, const Tab1D<T> *tab) {
         [&] {
           for (int r = 0; r < reps; ++r)
             launch_cell_apply<T>(R.d, tab, C->sym ? kApplyA | kApplySym : kApplyA, R.x, nullptr, R.r, nullptr, C->s,
-                                 R.shape, R.geo, R.rho);
+                                 R.shape, R.geo, R.geox, R.rho);
         },
         &ex[ci]);
   }
@@ -1598,7 +1606,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
       }
     }
     LevelDesc<double> d{};
-    double *geo_l = nullptr;
+    double *geo_l = nullptr, *geox_l = nullptr;
     d.dim = dim;
     d.k = k;
     for (int a = 0; a < 3; ++a) {
@@ -1699,6 +1707,11 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
         if ((st = dalloc(C, &geo_l, cells * per))) return st;
         launch_col_geometry<double>(d, geo_l, C->s);
         SMF_CUDA_OK(cudaGetLastError());
+        if (k == 2 && gbytes <= (long long)(free_b / 4)) {
+          if ((st = dalloc(C, &geox_l, fx_geometry_bytes(cells) / (long long)sizeof(double)))) return st;
+          launch_fx_geometry(d, geox_l, C->s);
+          SMF_CUDA_OK(cudaGetLastError());
+        }
       }
       // FP32 levels of at most 32^3 cells (56.6 MB for k = 2): stored as a candidate that the
       // setup's timing keeps or drops per level.  On the small levels a launch is a dependency
@@ -1715,6 +1728,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
     C->L64[l].d = d;
     C->L32[l].d = f;
     C->L64[l].geo = geo_l;
+    C->L64[l].geox = geox_l;
     if ((st = alloc_level_buffers(C, C->L64[l]))) return st;
     if ((st = alloc_level_buffers(C, C->L32[l]))) return st;
   }
@@ -3391,7 +3405,7 @@ int stokes_lift_rhs(stokes_ctx *C, const double *uD, double *b, void *stream) {
   // kx = [A B^T; B 0] u_D with the Dirichlet values read (rows of constrained DoFs stay zero)
   R.zero(L.kx, n);
   launch_cell_apply<double>(L.d, C->tab64, Runner<double>(C).form(kApplyA | kApplyBT | kApplyB | kApplyUnmasked), uD,
-                            uD + nu, L.kx, L.kx + nu, C->s, -1, nullptr, L.rho);
+                            uD + nu, L.kx, L.kx + nu, C->s, -1, nullptr, nullptr, L.rho);
   ++C->launches;
   R.vec(k_axpy<double>, n, b, -1.0, (const double *)L.kx, n);
   R.zero(L.kx, n);
@@ -3505,11 +3519,11 @@ int stokes_time_apply(stokes_ctx *C, int level, int precision, int blocks, int r
     if (precision == 64) {
       LevelRT<double> &R = C->L64[level];
       launch_cell_apply<double>(R.d, C->tab64, Runner<double>(C).form(blocks), R.x, R.x + R.d.n_u, R.r, R.r + R.d.n_u,
-                                C->s, R.shape, R.geo, R.rho, C->det ? &C->gb : nullptr);
+                                C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr);
     } else {
       LevelRT<float> &R = C->L32[level];
       launch_cell_apply<float>(R.d, C->tab32, Runner<float>(C).form(blocks), R.x, R.x + R.d.n_u, R.r, R.r + R.d.n_u,
-                               C->s, R.shape, R.geo, R.rho, C->det ? &C->gb : nullptr);
+                               C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr);
     }
     ++C->launches;
   }

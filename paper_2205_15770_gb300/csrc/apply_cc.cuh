@@ -16,6 +16,7 @@
 //     everywhere else), so the A block is 7 sweeps of 1D matrices over the nodal values and
 //     B, B^T are 3 sweeps each; no quadrature-point arrays, no shared memory.
 //   * Scatter by atomicAdd at the gather's indices; constrained DoFs read as 0 and not written.
+// The plain and fused FP64 launches of k = 2 run in fixed point instead (apply_fx.cuh).
 #pragma once
 #include <algorithm>
 
@@ -1065,14 +1066,20 @@ template <int K, typename T>
 int launch_cell_apply_cc_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp, const T *geo,
                            const GridBarrier *det, cudaStream_t s) {
   if (L.k != K || !cc_serves(L, geo)) return -1;
+  constexpr bool PLAIN = !(K == 2 && sizeof(T) == 8);  // apply_fx.cuh serves the plain FP64 launches of k = 2
+  if (!PLAIN && !det) return -1;
 #define SMF_CC_CASE(M)                                                                   \
   case M:                                                                                \
-    if (L.cartesian)                                                                     \
-      return det ? launch_cc_det_mode<K, T, M, true>(L, u, p, yu, yp, geo, *det, s)      \
-                 : (launch_cc_mode<K, T, M, true>(L, u, p, yu, yp, geo, s), 0);          \
-    if constexpr (K == 2)                                                                \
-      return det ? launch_cc_det_mode<K, T, M, false>(L, u, p, yu, yp, geo, *det, s)     \
-                 : (launch_cc_mode<K, T, M, false>(L, u, p, yu, yp, geo, s), 0);         \
+    if (L.cartesian) {                                                                   \
+      if (det) return launch_cc_det_mode<K, T, M, true>(L, u, p, yu, yp, geo, *det, s);  \
+      if constexpr (PLAIN) launch_cc_mode<K, T, M, true>(L, u, p, yu, yp, geo, s);       \
+      return 0;                                                                          \
+    }                                                                                    \
+    if constexpr (K == 2) {                                                              \
+      if (det) return launch_cc_det_mode<K, T, M, false>(L, u, p, yu, yp, geo, *det, s); \
+      if constexpr (PLAIN) launch_cc_mode<K, T, M, false>(L, u, p, yu, yp, geo, s);      \
+      return 0;                                                                          \
+    }                                                                                    \
     return -1;
   switch (mode) {
     SMF_CC_CASE(kApplyA)
@@ -1085,13 +1092,11 @@ int launch_cell_apply_cc_k(const LevelDesc<T> &L, int mode, const T *u, const T 
 #undef SMF_CC_CASE
 }
 
-// Fused smoothing applications on a level served by this kernel (k = 2); -1 otherwise.
+// Fused smoothing applications on a level served by this kernel (k = 2, FP32); -1 otherwise.
 template <int K, typename T>
 int launch_cell_apply_cc_fused_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp,
                                  const T *geo, const Fuse<T> &F, cudaStream_t s) {
-  if constexpr (K != 2) {
-    return -1;
-  } else {
+  {
     if (L.k != 2 || !cc_serves(L, geo)) return -1;
 #define SMF_CCF_CASE(M)                                                                                         \
   case M: {                                                                                                     \

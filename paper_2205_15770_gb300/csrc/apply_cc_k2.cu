@@ -14,7 +14,4 @@ template int upload_cc_tables<2>(const Tab1D<double> &, cudaStream_t);
 template int launch_cell_apply_cc_fused_k<2, float>(const LevelDesc<float> &, int, const float *, const float *,
                                                      float *, float *, const float *, const Fuse<float> &,
                                                      cudaStream_t);
-template int launch_cell_apply_cc_fused_k<2, double>(const LevelDesc<double> &, int, const double *,
-                                                      const double *, double *, double *, const double *,
-                                                      const Fuse<double> &, cudaStream_t);
 }  // namespace smf

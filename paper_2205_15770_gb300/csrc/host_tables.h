@@ -14,7 +14,7 @@ double tridiag_max_eig(const std::vector<double> &a, const std::vector<double> &
 
 template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
-                      cudaStream_t s, int shape, const T *geo = nullptr, const T *rho = nullptr,
+                      cudaStream_t s, int shape, const T *geo = nullptr, const T *geox = nullptr, const T *rho = nullptr,
                       const GridBarrier *det = nullptr);
 template <typename T>
 int launch_cell_diag(const LevelDesc<T> &L, const Tab1D<T> *tab, T *dAs, T *dSloc, T *dMp, cudaStream_t s,
@@ -49,6 +49,13 @@ inline bool cc_level_supported(int dim, int k, int cartesian, size_t elt) {
   if (cartesian) return k == 2 || k == 3;
   return k == 2;
 }
+// The fixed-point FP64 kernel (shape 5, k = 2; plain and, with F, fused launches): -1 for a level or mode
+// it does not serve.  geo: trilinear levels, the coefficients that launch_fx_geometry writes at setup
+// (fx_geometry_bytes(cells) bytes).
+int launch_cell_apply_fx(const LevelDesc<double> &L, int mode, const double *u, const double *p, double *yu, double *yp,
+                         const void *geo, const Fuse<double> *F, cudaStream_t s);
+long long fx_geometry_bytes(long long cells);
+void launch_fx_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
 template <int K, typename T>
 int launch_cell_apply_cc_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp, const T *geo,
                            const GridBarrier *det, cudaStream_t s);
