@@ -443,7 +443,8 @@ struct Runner {
   }
   void vmult(int l, const T *x, T *y, bool identity) {
     if (identity) {  // y = identity rows of x (0 elsewhere), then the cell kernel accumulates
-      vec(k_init_identity<T>, nu(l) + np(l), L[l].d, x, y);
+      launch_kernel(k_init_identity<T>, rows_grid(L[l].d, VW), dim3(kVecThreads), 0, s, L[l].d, x, y);
+      note();
       apply_nz(l, kApplyA | kApplyBT | kApplyB, x, x + nu(l), y, y + nu(l));
     } else {
       apply(l, kApplyA | kApplyBT | kApplyB, x, x + nu(l), y, y + nu(l));
@@ -2017,10 +2018,10 @@ static void krylov_post(stokes_ctx *C, cudaGraphConditionalHandle cond, bool set
   // w = K z_j: the conversion writes the operator's identity rows too (no separate k_init_identity)
   const LevelDesc<double> &Lt = C->L64[top].d;
   if (from_fp32)
-    launch_kernel(k_convert_to_slot_id<float>, dim3(nb), dim3(kVecThreads), 0, C->s, Lt,
+    launch_kernel(k_convert_to_slot_id<float>, rows_grid(Lt, 1), dim3(kVecThreads), 0, C->s, Lt,
                   (const float *)C->L32[top].x, C->zcur, C->Z, N, ctl, C->w);
   else
-    launch_kernel(k_convert_to_slot_id<double>, dim3(nb), dim3(kVecThreads), 0, C->s, Lt,
+    launch_kernel(k_convert_to_slot_id<double>, rows_grid(Lt, 1), dim3(kVecThreads), 0, C->s, Lt,
                   (const double *)C->L64[top].x, C->zcur, C->Z, N, ctl, C->w);
   R64.apply_nz(top, kApplyA | kApplyBT | kApplyB, C->zcur, C->zcur + Lt.n_u, C->w, C->w + Lt.n_u);
   R64.applyC(top, C->zcur + Lt.n_u, C->w + Lt.n_u, -1.0);

@@ -1,6 +1,7 @@
 // Vector kernels: Chebyshev-Jacobi recurrence (Sec. 3.3.1), residuals, precision
 // conversion, FP64 reductions for the Krylov loop and Lanczos, SplitMix64 start vectors.
 #pragma once
+#include <algorithm>
 #include <initializer_list>
 
 #include "common.cuh"
@@ -289,22 +290,70 @@ __global__ void k_convert_zero(const Tin *__restrict__ a, Tout *__restrict__ out
   }
 }
 
+// Grid of the kernels on for_rows: V entries a thread.
+template <typename T>
+inline dim3 rows_grid(const LevelDesc<T> &L, int V) {
+  return dim3((unsigned)vec_blocks((std::max(L.nv, L.n_p) + V - 1) / V), (unsigned)L.dim + 1);
+}
+// One space of [u | p] per blockIdx.y (dim velocity components, then the pressure), entries in 16-byte packs on y's
+// alignment with single entries at both ends; f(i, constrained) per entry, i the index in [u | p].  Bound by
+// memory: the node of a pack comes from two 32-bit divisions (a velocity component has less than 2^31 nodes: the
+// context's work vectors alone would take 876 GB) where one 64-bit division and remainder per entry and axis took
+// 7.8 us at 32^3 (Q2, FP32) and 87 us at 64^3 (Q3, FP32: 95 MB written, 1.1 TB/s); with packs 3.6 and 41 us.
+template <typename T, int V, typename Pack_, typename One>
+__device__ __forceinline__ void for_rows(const LevelDesc<T> &L, const void *y, Pack_ pack, One one) {
+  const int c = blockIdx.y;
+  const bool vel = c < L.dim;
+  const long long base = vel ? c * L.nv : L.n_u;
+  const unsigned n = (unsigned)(vel ? L.nv : L.n_p), N0 = (unsigned)L.N[0], N1 = (unsigned)L.N[1];
+  const unsigned mis = (unsigned)((reinterpret_cast<uintptr_t>(y) + base * sizeof(T)) % (V * sizeof(T))) / (unsigned)sizeof(T);
+  const unsigned head = min(n, mis ? V - mis : 0u), packs = (n - head) / V;
+  const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, dt = gridDim.x * blockDim.x;
+  auto fixed = [&](unsigned gx, unsigned gy, unsigned gz) {
+    return vel && vel_constrained(L.N, L.faces, L.dim, (int)gx, (int)gy, (int)gz);
+  };
+  for (unsigned j = t0; j < packs; j += dt) {
+    const unsigned i = head + j * V;
+    unsigned m = 0;
+    if (vel) {
+      unsigned r = i / N0, gx = i - r * N0, gz = r / N1, gy = r - gz * N1;
+      const bool inside = gx > 0 && gx + V < N0 && gy > 0 && gy + 1 < N1 && (L.dim < 3 || (gz > 0 && gz + 1 < (unsigned)L.N[2]));
+#pragma unroll
+      for (int k = 0; k < V && !inside; ++k) {
+        m |= fixed(gx, gy, gz) ? 1u << k : 0u;
+        if (++gx == N0) {
+          gx = 0;
+          if (++gy == N1) {
+            gy = 0;
+            ++gz;
+          }
+        }
+      }
+    }
+    pack(base + i, m);
+  }
+  const unsigned ends = n - packs * V;  // the entries before the first and after the last pack
+  for (unsigned t = t0; t < ends; t += dt) {
+    const unsigned i = t < head ? t : t + packs * V, r = i / N0, gz = r / N1;
+    one(base + i, fixed(i - r * N0, r - gz * N1, gz));
+  }
+}
+
 // y = x on constrained velocity DoFs (identity rows of K), 0 on every other entry of [u | p]:
 // the start of y = K x before the cell kernel accumulates into the free rows.
 template <typename T>
 __global__ void k_init_identity(const LevelDesc<T> L, const T *__restrict__ x, T *__restrict__ y) {
   pdl_enter();
-  SMF_GRID_LOOP(i, L.n_u + L.n_p) {
-    T v = T(0);
-    if (i < L.n_u) {
-      const long long node = i % L.nv;
-      const int gx = (int)(node % L.N[0]);
-      const long long r = node / L.N[0];
-      const int gy = (int)(r % L.N[1]), gz = (int)(r / L.N[1]);
-      if (vel_constrained(L.N, L.faces, L.dim, gx, gy, gz)) v = x[i];
-    }
-    y[i] = v;
-  }
+  constexpr int V = 16 / sizeof(T);
+  for_rows<T, V>(
+      L, y,
+      [&](long long i, unsigned m) {
+        Pack<T, V> r;
+#pragma unroll
+        for (int k = 0; k < V; ++k) r.v[k] = (m >> k & 1u) ? x[i + k] : T(0);
+        *reinterpret_cast<Pack<T, V> *>(y + i) = r;
+      },
+      [&](long long i, bool fixed) { y[i] = fixed ? x[i] : T(0); });
 }
 
 // zero constrained velocity entries
@@ -471,20 +520,14 @@ __global__ void k_convert_to_slot_id(const LevelDesc<double> L, const Tin *__res
                                      double *__restrict__ y) {
   pdl_enter();
   double *zj = Z + (long long)ctl[0] * ldz;
-  SMF_GRID_LOOP(i, L.n_u + L.n_p) {
+  auto one = [&](long long i, bool fixed) {
     const double v = (double)a[i];
     z[i] = v;
     zj[i] = v;
-    double yi = 0.0;
-    if (i < L.n_u) {
-      const long long node = i % L.nv;
-      const int gx = (int)(node % L.N[0]);
-      const long long r = node / L.N[0];
-      const int gy = (int)(r % L.N[1]), gz = (int)(r / L.N[1]);
-      if (vel_constrained(L.N, L.faces, L.dim, gx, gy, gz)) yi = v;
-    }
-    y[i] = yi;
-  }
+    y[i] = fixed ? v : 0.0;
+  };
+  // z_j's slot need not start on 16 bytes (odd vector lengths): single stores there, packs nowhere
+  for_rows<double, 1>(L, y, [&](long long i, unsigned m) { one(i, m != 0); }, one);
 }
 
 }  // namespace smf
