@@ -121,8 +121,11 @@ int launch_cell_diag<double>(const LevelDesc<double> &L, const Tab1D<double> *ta
 
 // x = Kinv b on the coarse level: one warp per row, FP64 accumulation.
 template <typename T>
-__global__ void k_coarse_apply(const double *__restrict__ Kinv, int n0, const T *__restrict__ b, T *__restrict__ x) {
+__global__ void k_coarse_apply(const double *__restrict__ Kinv, int n0, const T *__restrict__ b, T *__restrict__ x,
+                               long long ld) {
   pdl_enter();
+  b = column(b, ld);
+  x = column(x, ld);
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= n0) return;
   const double *row = Kinv + (long long)warp * n0;
@@ -130,6 +133,42 @@ __global__ void k_coarse_apply(const double *__restrict__ Kinv, int n0, const T 
   for (int j = lane; j < n0; j += 32) s += row[j] * (double)b[j];
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) x[warp] = (T)s;
+}
+
+// ---- explicit cycle of a small level (setup_explicit) --------------------------------------------
+// x = M b, M n x n with rows of ldm entries (16-byte multiples, the padding zero): one warp per row, every
+// 16-byte piece of the row in flight.  Bound by the matrix read from L2: 2,312 rows (21 MB)
+// take 5 us, 2,467 rows 5.8 us.
+constexpr int kExplicitWarps = 16;
+__global__ void __launch_bounds__(32 * kExplicitWarps)
+    k_explicit_apply(const float *__restrict__ M, int n, int ldm, const float *__restrict__ b, float *__restrict__ x) {
+  pdl_enter();
+  const int row = blockIdx.x * kExplicitWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= n) return;
+  const float4 *m = reinterpret_cast<const float4 *>(M + (long long)row * ldm), *v = reinterpret_cast<const float4 *>(b);
+  const int full = n / 4;
+  float s[4] = {};
+#pragma unroll 8
+  for (int j = lane; j < full; j += 32) {
+    const float4 a = __ldg(m + j), c = v[j];
+    s[0] += a.x * c.x;
+    s[1] += a.y * c.y;
+    s[2] += a.z * c.z;
+    s[3] += a.w * c.w;
+  }
+  float t = (s[0] + s[1]) + (s[2] + s[3]);
+  const int j = 4 * full + lane;
+  if (j < n) t += M[(long long)row * ldm + j] * b[j];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+  if (lane == 0) x[row] = t;
+}
+// unit vectors j0 + column of length n
+__global__ void k_unit_cols(float *b, int n, int j0, long long ld) {
+  SMF_GRID_LOOP(i, n) b[blockIdx.y * ld + i] = i == j0 + (int)blockIdx.y ? 1.f : 0.f;
+}
+// column j0 + blockIdx.y of M
+__global__ void k_explicit_store(const float *x, int n, int j0, long long ld, float *M, int ldm) {
+  SMF_GRID_LOOP(i, n) M[i * ldm + j0 + blockIdx.y] = x[blockIdx.y * ld + i];
 }
 
 // x[i * stride] += s
@@ -275,6 +314,9 @@ struct stokes_ctx {
   bool use_graphs = true;
   bool fuse = true;  // fused smoothing where eligible (STOKES_NO_FUSE=1: the unfused path)
   GraphSlot g32[2], g64[2];  // [x_zero]
+  // FP32 cycle of level le from a zero start as an explicit matrix (setup_explicit; -1: none)
+  int le = -1, ldm = 0;
+  float *Mx = nullptr;
   // FGMRES with the Arnoldi state on the device: one graph (conditional while node over the inner
   // iterations of a restart cycle) replayed per cycle; kry_mode -1 not built yet, 0 host-driven
   // loop (STOKES_HOST_KRYLOV=1, or conditional graph nodes unavailable), 1 device loop
@@ -369,7 +411,12 @@ struct Runner {
   cudaStream_t s;
   std::vector<LevelRT<T>> &L;
   const Tab1D<T> *tab;
+  int cols = 1;      // vectors handled by every launch, ld entries apart (setup_explicit; FP32, unfused forms)
+  long long ld = 0;
   explicit Runner(stokes_ctx *c) : C(c), s(c->s), L(levels<T>(c)), tab(tables<T>(c)) {}
+  // several columns on their own work vectors
+  Runner(stokes_ctx *c, std::vector<LevelRT<T>> &levels_, int cols_, long long ld_)
+      : C(c), s(c->s), L(levels_), tab(tables<T>(c)), cols(cols_), ld(ld_) {}
   // launches on the caller's stream (which may be the default stream 0)
   struct OnStream {};
   Runner(stokes_ctx *c, cudaStream_t stream, OnStream) : C(c), s(stream), L(levels<T>(c)), tab(tables<T>(c)) {}
@@ -385,7 +432,7 @@ struct Runner {
   long long np(int l) const { return L[l].d.n_p; }
   template <typename... KA, typename... A>
   void vec(void (*k)(KA...), long long n, A... args) {
-    launch_kernel(k, dim3(vec_blocks(n)), dim3(kVecThreads), 0, s, args...);
+    launch_kernel(k, dim3(vec_blocks(n), cols), dim3(kVecThreads), 0, s, args...);
     note();
   }
   // Packed launch: kv processes 16-byte packs (VW elements), k1 single elements; kv is chosen
@@ -394,9 +441,9 @@ struct Runner {
   template <typename K1, typename KV, typename... A>
   void vecp(K1 k1, KV kv, std::initializer_list<const void *> ptrs, long long n, A... args) {
     if (all_aligned(16, ptrs))
-      launch_kernel(kv, dim3(vec_blocks((n + VW - 1) / VW)), dim3(kVecThreads), 0, s, args...);
+      launch_kernel(kv, dim3(vec_blocks((n + VW - 1) / VW), cols), dim3(kVecThreads), 0, s, args...);
     else
-      launch_kernel(k1, dim3(vec_blocks(n)), dim3(kVecThreads), 0, s, args...);
+      launch_kernel(k1, dim3(vec_blocks(n), cols), dim3(kVecThreads), 0, s, args...);
     note();
   }
 
@@ -436,6 +483,17 @@ struct Runner {
       o.out[1] = fp(yp);
       o.items = pq_items(o);
       return;
+    }
+    if constexpr (std::is_same<T, float>::value) {
+      if (cols > 1) {
+        switch (L[l].d.k) {
+          case 2: launch_cell_apply_cols_k<2, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
+          case 3: launch_cell_apply_cols_k<3, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
+          default: launch_cell_apply_cols_k<4, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
+        }
+        note();
+        return;
+      }
     }
     launch_cell_apply<T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].shape, L[l].geo, L[l].geox, L[l].rho,
                          C->det ? &C->gb : nullptr);
@@ -522,7 +580,7 @@ struct Runner {
       return;
     }
     vecp(k_cheb_init<T, 1>, k_cheb_init<T, VW>, {a, b, Dinv, r_out, d, x, base, final_out, acc_out, za, zb}, n, a, b,
-         sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb, n);
+         sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb, n, ld);
   }
   void cheb_step_op(int l, long long n, const T *r, T *t, const T *Dinv, T c1, T c2, T *d, T *x, const T *base,
                     T fscale, T *final_out, T *acc_out) {
@@ -542,7 +600,7 @@ struct Runner {
       return;
     }
     vecp(k_cheb_step<T, 1>, k_cheb_step<T, VW>, {r, t, Dinv, d, x, base, final_out, acc_out}, n, r, t, Dinv, c1, c2,
-         d, x, base, fscale, final_out, acc_out, n);
+         d, x, base, fscale, final_out, acc_out, n, ld);
   }
   // y = B A^-1_hat B^T q   (y zero on entry)
   void S_tilde(int l, const T *q, T *y) {
@@ -581,7 +639,8 @@ struct Runner {
       o.items = pq_items(o);
       return;
     }
-    launch_kernel(k_coarse_apply<T>, dim3((n0 * 32 + 255) / 256), dim3(256), 0, s, (const double *)C->Kinv, n0, b, x);
+    launch_kernel(k_coarse_apply<T>, dim3((n0 * 32 + 255) / 256, cols), dim3(256), 0, s, (const double *)C->Kinv, n0, b, x,
+                  ld);
     note();
   }
   // restriction out = P^T in, or P^T (in - sub) (the residual formed while restricting)
@@ -601,14 +660,14 @@ struct Runner {
     }
     if (sub) {
       if (n < 32768)
-        vec(k_restrict<T, W, 8, true>, n * 8, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub);
+        vec(k_restrict<T, W, 8, true>, n * 8, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub, ld);
       else
-        vec(k_restrict<T, W, 1, true>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub);
+        vec(k_restrict<T, W, 1, true>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub, ld);
     } else {
       if (n < 32768)
-        vec(k_restrict<T, W, 8, false>, n * 8, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub);
+        vec(k_restrict<T, W, 8, false>, n * 8, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub, ld);
       else
-        vec(k_restrict<T, W, 1, false>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub);
+        vec(k_restrict<T, W, 1, false>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, zero_c, sub, ld);
     }
   }
   void restrict_to(int lf, const T *in, T *out, T *zero_c, const T *sub = nullptr) {
@@ -634,9 +693,9 @@ struct Runner {
       return;
     }
     switch (L[lf].d.k) {
-      case 2: vec(k_prolongate<T, 9>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf); break;
-      case 3: vec(k_prolongate<T, 13>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf); break;
-      default: vec(k_prolongate<T, 17>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf); break;
+      case 2: vec(k_prolongate<T, 9>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf, ld); break;
+      case 3: vec(k_prolongate<T, 13>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf, ld); break;
+      default: vec(k_prolongate<T, 17>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf, ld); break;
     }
   }
   // ---- fused smoothing: k_A = 1, 3D column kernel ------------------------------------------
@@ -650,7 +709,7 @@ struct Runner {
   // step, residual) or written by k_fused_finish.
   bool fused_ok(int l) const { return fused_eligible(l) && L[l].fuse; }
   bool fused_eligible(int l) const {
-    return C->fuse && !C->det && !hasC() && !C->sym && !L[l].rho && C->o.kA == 1 && C->o.kS >= 1 && C->o.kS <= 4 &&
+    return cols == 1 && C->fuse && !C->det && !hasC() && !C->sym && !L[l].rho && C->o.kA == 1 && C->o.kS >= 1 && C->o.kS <= 4 &&
            L[l].d.dim == 3 && L[l].shape >= 0;
   }
   T *pairU(int l, int pr) { return pr == 0 ? L[l].tu : L[l].cx; }
@@ -853,6 +912,21 @@ struct Runner {
     if (pend >= 0) fused_finish(l, x, pend);
   }
 
+  // The gamma recursive calls of Algorithm 1 on level l, x_l from zero (the restriction zeroed it), or their
+  // explicit matrix.
+  void coarse_cycles(int l) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (l == C->le && cols == 1 && !rec()) {
+        const int n = (int)(nu(l) + np(l));
+        launch_kernel(k_explicit_apply, dim3((n + kExplicitWarps - 1) / kExplicitWarps), dim3(32 * kExplicitWarps), 0, s,
+                      (const float *)C->Mx, n, C->ldm, (const float *)L[l].b, L[l].x);
+        note();
+        return;
+      }
+    }
+    const int gam = C->o.cycle == 1 ? 2 : 1;
+    for (int j = 0; j < gam; ++j) cycle(l, L[l].x, L[l].b, j == 0);
+  }
   // Algorithm 1: MG(x_l, b_l) with gamma = 1 (V) or 2 (W); returns after the coarse solve on l = 0.
   void cycle(int l, T *x, const T *b, bool x_zero) {
     if (l == 0) {
@@ -881,8 +955,7 @@ struct Runner {
       applyC(l, x + nu(l), R.kx + nu(l), T(-1));
       restrict_to(l, b, L[l - 1].b, L[l - 1].x, R.kx);
     }
-    const int gam = C->o.cycle == 1 ? 2 : 1;
-    for (int j = 0; j < gam; ++j) cycle(l - 1, L[l - 1].x, L[l - 1].b, j == 0);
+    coarse_cycles(l - 1);
     prolongate(l, L[l - 1].x, x, 1, pend >= 0 ? pairU(l, pend) : nullptr, pend >= 0 ? pairT(l, pend) : nullptr,
                kx_used ? R.kx : nullptr);
     pend = -1;
@@ -1423,6 +1496,69 @@ static int autotune_fusion(stokes_ctx *C, int l) {
   return zero_level_work(C, L);
 }
 
+// The FP32 cycle of a small level below the finest as an explicit matrix.  From a zero start the gamma
+// recursive calls are linear in the right-hand side, x_l = M b_l, and on a small level their ~40 (2D: per
+// level) dependent launches of 2-4 us cost far more than reading M: 4^3 and the 2^3 coarse solve 130-156 us
+// against 5 us for M's 21 MB, which stay in L2; three 2D levels up to 16^2 460 us against 6.  So the largest level l <= n_levels - 2 whose M takes at
+// most kExplicitBytes becomes explicit (FP32 multigrid, C = 0, not in deterministic mode: M is summed by
+// atomics).  The line: a matrix of 48 MB, 3,464 unknowns, is read in 6 us and built in about 10 ms; at twice
+// the unknowns (6^3 cells: 192 MB, beyond L2) the build is four times as long and the read 30 us.
+// M's columns are the cycle of the unit vectors, kExplicitCols of them in every launch (column()).
+// STOKES_NO_EXPLICIT=1 keeps the launches.
+constexpr long long kExplicitBytes = 48ll << 20;
+constexpr int kExplicitCols = 512;
+static int setup_explicit(stokes_ctx *C) {
+  const char *off = getenv("STOKES_NO_EXPLICIT");
+  if (!C->o.vcycle_fp32 || C->det || C->c_mass != 0.0 || C->c_grad != 0.0 || (off && off[0] == '1')) return STOKES_OK;
+  int le = -1;
+  for (int l = 1; l <= C->nl - 2; ++l) {
+    const long long n = C->L32[l].d.n_u + C->L32[l].d.n_p;
+    if (n * (n + 3) / 4 * 4 * (long long)sizeof(float) <= kExplicitBytes) le = l;
+  }
+  if (le < 1) return STOKES_OK;
+  const int n = (int)(C->L32[le].d.n_u + C->L32[le].d.n_p), ldm = (n + 3) / 4 * 4;
+  int st;
+  float *M = nullptr;
+  if ((st = dalloc(C, &M, (long long)n * ldm))) return st;
+  // work vectors of levels 0 .. le for a batch of columns, every column of every vector ld entries apart
+  const int cols = std::min(n, kExplicitCols);
+  const long long ld = (n + 63) / 64 * 64;
+  std::vector<LevelRT<float>> Lb(C->L32.begin(), C->L32.begin() + le + 1);
+  constexpr int NB = 20;
+  float *mem = nullptr;
+  const size_t bytes = (size_t)(le + 1) * NB * cols * ld * sizeof(float);
+  if (cudaMalloc((void **)&mem, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return STOKES_OK;  // no room: the launches stay
+  }
+  cudaMemsetAsync(mem, 0, bytes, C->s);
+  float *p = mem;
+  for (LevelRT<float> &R : Lb) {
+    float **v[NB] = {&R.x,  &R.b,   &R.kx,  &R.tu,  &R.ru, &R.uhat, &R.cx, &R.cd, &R.ct, &R.r2,
+                     &R.cx2, &R.cd2, &R.ct2, &R.au, &R.pt, &R.rp,   &R.px, &R.pd, &R.ps, &R.dp};
+    for (float **q : v) {
+      *q = p;
+      p += (long long)cols * ld;
+    }
+  }
+  for (int j0 = 0; j0 < n; j0 += cols) {
+    const int nc = std::min(cols, n - j0);
+    Runner<float> R(C, Lb, nc, ld);
+    cudaMemsetAsync(Lb[le].x, 0, (size_t)cols * ld * sizeof(float), C->s);
+    k_unit_cols<<<dim3(vec_blocks(n), nc), kVecThreads, 0, C->s>>>(Lb[le].b, n, j0, ld);
+    R.coarse_cycles(le);
+    k_explicit_store<<<dim3(vec_blocks(n), nc), kVecThreads, 0, C->s>>>(Lb[le].x, n, j0, ld, M, ldm);
+  }
+  const cudaError_t e = cudaStreamSynchronize(C->s);
+  cudaFree(mem);
+  SMF_CUDA_OK(e);
+  SMF_CUDA_OK(cudaGetLastError());
+  C->Mx = M;
+  C->ldm = ldm;
+  C->le = le;
+  return STOKES_OK;
+}
+
 // STOKES_TUNING="s32=a,b,..;s64=..;f32=..;f64=..[;g32=..]" replaces the setup's timings: launch
 // shapes (1, 3, 4, -1 or 5) and smoother forms (1 fused, 0 unfused) per level, coarsest first, for
 // FP32 and FP64, and optionally whether the FP32 column kernels read the stored per-point geometry
@@ -1923,6 +2059,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
       }
     }
   }
+  if ((st = setup_explicit(C))) return st;
   SMF_CUDA_OK(cudaStreamSynchronize(C->s));
   SMF_CUDA_OK(cudaGetLastError());
   if (C->det) {

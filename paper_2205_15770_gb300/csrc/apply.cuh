@@ -157,8 +157,12 @@ template <int DIM, int K, typename T, bool CART>
 __global__ void __launch_bounds__(CellShape<DIM, K>::THREADS)
     stokes_cell_apply(const LevelDesc<T> L, const Tab1D<T> *__restrict__ tab, const int mode,
                       const T *__restrict__ u, const T *__restrict__ p, T *__restrict__ yu,
-                      T *__restrict__ yp, const T *__restrict__ rho_cell) {
+                      T *__restrict__ yp, const T *__restrict__ rho_cell, const long long ld) {
   pdl_enter();
+  u = column(u, ld);
+  p = column(p, ld);
+  yu = column(yu, ld);
+  yp = column(yp, ld);
   using CS = CellShape<DIM, K>;
   constexpr int NQ = CS::NQ, NV = CS::NV, NPR = CS::NPR, NP = CS::NP, NPP = CS::NPP;
   extern __shared__ __align__(16) unsigned char smem_raw[];

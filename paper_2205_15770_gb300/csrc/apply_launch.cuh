@@ -21,12 +21,12 @@ static inline bool getenv_generic() {
 
 template <int DIM, int K, typename T, bool CART>
 static int launch_apply_dim(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu,
-                            T *yp, cudaStream_t s, const T *rho) {
+                            T *yp, cudaStream_t s, const T *rho, int cols = 1, long long ld = 0) {
   using CS = CellShape<DIM, K>;
   const long long blocks = (L.n_cells + CS::CPB - 1) / CS::CPB;
   const size_t smem = sizeof(Tab1D<T>) + (size_t)CS::CPB * CS::PER_CELL * sizeof(T);
-  launch_kernel(stokes_cell_apply<DIM, K, T, CART>, dim3((unsigned)blocks), dim3(CS::THREADS), smem, s, L, tab, mode, u,
-                p, yu, yp, rho);
+  launch_kernel(stokes_cell_apply<DIM, K, T, CART>, dim3((unsigned)blocks, (unsigned)cols), dim3(CS::THREADS), smem, s, L,
+                tab, mode, u, p, yu, yp, rho, ld);
   return 0;
 }
 
@@ -84,6 +84,17 @@ int launch_cell_apply_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, co
                        : launch_apply_dim<3, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho);
   return L.cartesian ? launch_apply_dim<2, K, T, true>(L, tab, mode, u, p, yu, yp, s, rho)
                      : launch_apply_dim<2, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho);
+}
+
+// The same applications on `cols` vectors at once, ld entries apart, in the point kernel.
+template <int K, typename T>
+int launch_cell_apply_cols_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
+                             cudaStream_t s, const T *rho, int cols, long long ld) {
+  if (L.dim == 3)
+    return L.cartesian ? launch_apply_dim<3, K, T, true>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld)
+                       : launch_apply_dim<3, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld);
+  return L.cartesian ? launch_apply_dim<2, K, T, true>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld)
+                     : launch_apply_dim<2, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld);
 }
 
 template <int DIM, int K, typename T, bool CART>
@@ -224,6 +235,9 @@ int launch_cell_diag_k(const LevelDesc<T> &L, const Tab1D<T> *tab, T *dAs, T *dS
   template int launch_cell_apply_k<KK, double>(const LevelDesc<double> &, const Tab1D<double> *, int,          \
                                                 const double *, const double *, double *, double *,            \
                                                 cudaStream_t, int, const double *, const double *);                                             \
+  template int launch_cell_apply_cols_k<KK, float>(const LevelDesc<float> &, const Tab1D<float> *, int,        \
+                                                    const float *, const float *, float *, float *,           \
+                                                    cudaStream_t, const float *, int, long long);               \
   template int launch_cell_apply_fused_k<KK, float>(const LevelDesc<float> &, int, const float *, const float *, \
                                                      float *, float *, cudaStream_t, int, const Fuse<float> &,       \
                                                      const float *);   \

@@ -125,6 +125,13 @@ struct GridBarrier {
   void *loc32 = nullptr, *loc64 = nullptr;
 };
 #if defined(__CUDACC__)
+// Launches over several columns at once (the setup of the explicit small-level cycle): blockIdx.y is the
+// column, every vector's columns are ld entries apart.  One column: gridDim.y = 1.
+template <typename T>
+__device__ __forceinline__ T *column(T *p, long long ld) {
+  return p ? p + blockIdx.y * ld : p;
+}
+
 // Input loads of the kernels: plain (the compiler may use the read-only path) or, in the
 // persistent work-queue kernel whose inputs are written by earlier work items of the same launch,
 // L2 loads that bypass the per-SM caches (COH).  (L1-cached loads after the acquire fence measured

@@ -16,6 +16,10 @@ template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
                       cudaStream_t s, int shape, const T *geo = nullptr, const T *geox = nullptr, const T *rho = nullptr,
                       const GridBarrier *det = nullptr);
+// `cols` vectors at once, ld entries apart (FP32)
+template <int K, typename T>
+int launch_cell_apply_cols_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
+                             cudaStream_t s, const T *rho, int cols, long long ld);
 template <typename T>
 int launch_cell_diag(const LevelDesc<T> &L, const Tab1D<T> *tab, T *dAs, T *dSloc, T *dMp, cudaStream_t s,
                      const T *rho, int sym);

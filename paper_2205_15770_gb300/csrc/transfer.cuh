@@ -84,8 +84,12 @@ __device__ __forceinline__ T restrict_terms(const LevelDesc<T> &F, const LevelDe
 // fill the GPU).
 template <typename T, int W, int LANES, bool SUB = false>
 __global__ void k_restrict(const LevelDesc<T> F, const LevelDesc<T> C, const XferTabs<T> X, const T *__restrict__ in,
-                           T *__restrict__ out, T *__restrict__ zero_c, const T *__restrict__ minus = nullptr) {
+                           T *__restrict__ out, T *__restrict__ zero_c, const T *__restrict__ minus, long long ld) {
   pdl_enter();
+  in = column(in, ld);
+  out = column(out, ld);
+  zero_c = column(zero_c, ld);
+  minus = column(minus, ld);
   const long long total = (C.n_u + C.n_p) * LANES;
   const int sub = threadIdx.x & (LANES - 1);
   // the loop condition depends only on the warp's first index, so all 32 lanes iterate together
@@ -136,8 +140,13 @@ __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDes
 template <typename T, int W>
 __global__ void k_prolongate(const LevelDesc<T> F, const LevelDesc<T> C, const XferTabs<T> X, const T *__restrict__ in,
                              T *__restrict__ out, int add, T *__restrict__ z0, T *__restrict__ z1,
-                             T *__restrict__ zf = nullptr) {
+                             T *__restrict__ zf, long long ld) {
   pdl_enter();
+  in = column(in, ld);
+  out = column(out, ld);
+  z0 = column(z0, ld);
+  z1 = column(z1, ld);
+  zf = column(zf, ld);
   SMF_GRID_LOOP(i, F.n_u + F.n_p) {
     const bool vel = i < F.n_u;
     if (zf) zf[i] = T(0);

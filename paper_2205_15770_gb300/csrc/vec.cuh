@@ -197,8 +197,19 @@ __device__ __forceinline__ void cheb_init_packj(long long j, const T *a, const T
 template <typename T, int V>
 __global__ void k_cheb_init(const T *a, const T *b, T sr, const T *__restrict__ Dinv,
                             T c0, T *__restrict__ r_out, T *__restrict__ d, T *__restrict__ x, const T *__restrict__ base,
-                            T fscale, T *__restrict__ final_out, T *__restrict__ acc_out, T *za, T *zb, long long n) {
+                            T fscale, T *__restrict__ final_out, T *__restrict__ acc_out, T *za, T *zb, long long n,
+                            long long ld) {
   pdl_enter();
+  a = column(a, ld);
+  b = column(b, ld);
+  r_out = column(r_out, ld);
+  d = column(d, ld);
+  x = column(x, ld);
+  base = column(base, ld);
+  final_out = column(final_out, ld);
+  acc_out = column(acc_out, ld);
+  za = column(za, ld);
+  zb = column(zb, ld);
   SMF_PACK_LOOP(j, n, V)
   cheb_init_packj<T, V>(j, a, b, sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb);
   SMF_TAIL_LOOP(i, n, V) cheb_init_elem(i, a, b, sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb);
@@ -238,8 +249,15 @@ __device__ __forceinline__ void cheb_step_packj(long long j, const T *r, T *t, c
 template <typename T, int V>
 __global__ void k_cheb_step(const T *__restrict__ r, T *__restrict__ t, const T *__restrict__ Dinv, T c1, T c2,
                             T *__restrict__ d, T *__restrict__ x, const T *__restrict__ base, T fscale,
-                            T *__restrict__ final_out, T *__restrict__ acc_out, long long n) {
+                            T *__restrict__ final_out, T *__restrict__ acc_out, long long n, long long ld) {
   pdl_enter();
+  r = column(r, ld);
+  t = column(t, ld);
+  d = column(d, ld);
+  x = column(x, ld);
+  base = column(base, ld);
+  final_out = column(final_out, ld);
+  acc_out = column(acc_out, ld);
   SMF_PACK_LOOP(j, n, V) cheb_step_packj<T, V>(j, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out);
   SMF_TAIL_LOOP(i, n, V) cheb_step_elem(i, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out);
 }
