@@ -698,7 +698,7 @@ struct Runner {
       default: vec(k_prolongate<T, 17>, n, L[lf].d, L[lf - 1].d, L[lf].xf, in, out, add, z0, z1, zf, ld); break;
     }
   }
-  // ---- fused smoothing: k_A = 1, 3D column kernel ------------------------------------------
+  // ---- fused smoothing: k_A = 1 ------------------------------------------
   // The Chebyshev-Jacobi and Uzawa vector updates of smooth_step are folded into the gathers of
   // the cell-kernel applications (Fuse descriptors), so a step is 5 + 3 k_S launches instead of
   // 10 + 6 k_S.  Work buffers: two velocity pairs (TU: B^T / A|B^T target, T: A target) used
@@ -710,7 +710,7 @@ struct Runner {
   bool fused_ok(int l) const { return fused_eligible(l) && L[l].fuse; }
   bool fused_eligible(int l) const {
     return cols == 1 && C->fuse && !C->det && !hasC() && !C->sym && !L[l].rho && C->o.kA == 1 && C->o.kS >= 1 && C->o.kS <= 4 &&
-           L[l].d.dim == 3 && L[l].shape >= 0;
+           L[l].shape >= 0;
   }
   T *pairU(int l, int pr) { return pr == 0 ? L[l].tu : L[l].cx; }
   T *pairT(int l, int pr) { return pr == 0 ? L[l].ct : L[l].ct2; }

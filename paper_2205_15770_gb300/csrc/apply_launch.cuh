@@ -3,6 +3,7 @@
 #include <cstdlib>
 #include "apply.cuh"
 #include "apply_col.cuh"
+#include "apply_2d.cuh"
 #include "apply_c.cuh"
 #include "vec.cuh"
 #include "host_tables.h"
@@ -79,6 +80,9 @@ int launch_cell_apply_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, co
       default: break;
     }
   }
+  if (L.dim == 2 && !getenv_generic() && shape >= 0 && !generic_a &&
+      launch_2d<K, T, false>(L, mode, u, p, yu, yp, s, Fuse<T>{}) == 0)
+    return 0;
   if (L.dim == 3)
     return L.cartesian ? launch_apply_dim<3, K, T, true>(L, tab, mode, u, p, yu, yp, s, rho)
                        : launch_apply_dim<3, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho);
@@ -160,12 +164,13 @@ int launch_col_geometry_k(const LevelDesc<T> &L, T *geo, cudaStream_t s) {
   return 0;
 }
 
-// Fused application (3D column kernel only; shape >= 0): returns -1 for a mode without a fused
-// instantiation so that the caller can reject it.
+// Fused application (3D: column kernel; 2D: its one kernel; shape >= 0): returns -1 for a mode without a
+// fused instantiation so that the caller can reject it.
 template <int K, typename T>
 int launch_cell_apply_fused_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp, cudaStream_t s,
                               int shape, const Fuse<T> &F, const T *geo) {
-  if (L.dim != 3 || shape < 0) return -1;
+  if (shape < 0) return -1;
+  if (L.dim == 2) return launch_2d<K, T, true>(L, mode, u, p, yu, yp, s, F);
   switch (mode) {
     case kApplyA: return launch_col_mode<K, T, kApplyA, true>(L, u, p, yu, yp, s, shape, F, geo);
     case kApplyBT: return launch_col_mode<K, T, kApplyBT, true>(L, u, p, yu, yp, s, shape, F, geo);
