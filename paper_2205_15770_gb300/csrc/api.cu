@@ -52,7 +52,7 @@ int cuda_fail(cudaError_t e, const char *what, const char *file, int line) {
 
 template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
-                      cudaStream_t s, int shape, const T *geo, const T *geox, const T *rho, const GridBarrier *det) {
+                      cudaStream_t s, int shape, const T *geo, const T *geox, const T *rho, const GridBarrier *det, bool plane) {
   if (shape == 5 || det) {
     // cell-component kernel (Laplacian form, constant rho); the column kernel serves the rest.
     // det: its deterministic cooperative form (setup admits deterministic mode only where it serves
@@ -61,6 +61,8 @@ int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, cons
     if (!generic_a) {
       if constexpr (sizeof(T) == 8) {
         if (!det && launch_cell_apply_fx(L, mode, u, p, yu, yp, geox, nullptr, s) == 0) return 0;
+      } else {
+        if (!det && plane && launch_cell_apply_pl(L, mode, u, p, yu, yp, geox, nullptr, s) == 0) return 0;
       }
       const int r = L.k == 2 ? launch_cell_apply_cc_k<2, T>(L, mode, u, p, yu, yp, geo, det, s)
                              : (L.k == 3 ? launch_cell_apply_cc_k<3, T>(L, mode, u, p, yu, yp, geo, det, s) : -1);
@@ -221,7 +223,8 @@ struct LevelRT {
   bool fuse = true;  // fused smoothing on this level (set by the setup's timing, when eligible)
   const T *geo = nullptr;  // 3D trilinear: precomputed per-point geometry the column kernel reads
   const T *geo_stored = nullptr;  // FP32: the stored geometry, used (geo) where the setup's timing keeps it
-  const T *geox = nullptr; // FP64, k = 2, trilinear: the fixed-point form's digits of it
+  const T *geox = nullptr; // k = 2, trilinear: the stored coefficients of shape 5's plane kernels (apply_fx.cuh, apply_pl.cuh)
+  bool plane = false;      // FP32 shape 5: the plane kernel (false: the cell-component kernel)
   const T *rho = nullptr;  // per-cell density of the gamma rho mass term (null: rho = 1)
   const T *Ce = nullptr;   // packed element matrices of the stabilisation block C (null: on the fly)
   T *DAinv = nullptr, *DSinv = nullptr;
@@ -496,7 +499,7 @@ struct Runner {
       }
     }
     launch_cell_apply<T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].shape, L[l].geo, L[l].geox, L[l].rho,
-                         C->det ? &C->gb : nullptr);
+                         C->det ? &C->gb : nullptr, L[l].plane);
     note();
   }
   void vmult(int l, const T *x, T *y, bool identity) {
@@ -724,6 +727,8 @@ struct Runner {
       int r;
       if constexpr (sizeof(T) == 8)
         r = launch_cell_apply_fx(L[l].d, mode, u, p, yu, yp, L[l].geox, &F, s);
+      else if (L[l].plane)
+        r = launch_cell_apply_pl(L[l].d, mode, u, p, yu, yp, L[l].geox, &F, s);
       else
         r = launch_cell_apply_cc_fused_k<2, T>(L[l].d, mode, u, p, yu, yp, L[l].geo, F, s);
       if (r == 0) {
@@ -1399,11 +1404,12 @@ static int autotune_level(stokes_ctx *C, LevelRT<T> &R, const Tab1D<T> *tab) {
                   (R.d.cartesian || sizeof(T) == 4 || R.geox);
   const bool sg = R.geo_stored && !R.geo;
   // candidates: column shapes 4, 1, 3 (on-the-fly geometry), point kernel, cell-component kernel,
-  // then the column shapes reading the stored geometry
-  constexpr int NMAX = 8;
-  const int cands[NMAX] = {4, 1, 3, -1, 5, 4, 1, 3};
-  const bool cgeo[NMAX] = {false, false, false, false, false, true, true, true};
-  bool use[NMAX] = {true, true, true, true, cc, sg, sg, sg};
+  // then the column shapes reading the stored geometry, and the plane form of shape 5 (FP32, k = 2)
+  constexpr int NMAX = 9;
+  const int cands[NMAX] = {4, 1, 3, -1, 5, 4, 1, 3, 5};
+  const bool cgeo[NMAX] = {false, false, false, false, false, true, true, true, false};
+  const bool pl = R.plane && cc;  // shape 5 has a plane form too (the last candidate)
+  bool use[NMAX] = {true, true, true, true, cc, sg, sg, sg, pl};
   const int reps = sizeof(T) == 8 ? 3 : 20, rounds = 3;
   cudaEvent_t e0, e1;
   SMF_CUDA_OK(cudaEventCreate(&e0));
@@ -1416,13 +1422,14 @@ static int autotune_level(stokes_ctx *C, LevelRT<T> &R, const Tab1D<T> *tab) {
   for (int ci = 0; ci < NMAX && st == STOKES_OK; ++ci) {
     if (!use[ci]) continue;
     R.shape = cands[ci];
+    R.plane = pl && ci == NMAX - 1;
     R.geo = cgeo[ci] ? R.geo_stored : geo0;
     st = capture_graph(
         C,
         [&] {
           for (int r = 0; r < reps; ++r)
             launch_cell_apply<T>(R.d, tab, C->sym ? kApplyA | kApplySym : kApplyA, R.x, nullptr, R.r, nullptr, C->s,
-                                 R.shape, R.geo, R.geox, R.rho);
+                                 R.shape, R.geo, R.geox, R.rho, nullptr, R.plane);
         },
         &ex[ci]);
   }
@@ -1444,6 +1451,7 @@ static int autotune_level(stokes_ctx *C, LevelRT<T> &R, const Tab1D<T> *tab) {
   for (int ci = 1; ci < NMAX; ++ci)
     if (use[ci] && best[ci] < 0.97f * best[choice]) choice = ci;
   R.shape = cands[choice];
+  R.plane = pl && !(use[4] && choice == 4);  // kept for a later set_launch_shape unless the cell-component form won
   int fc = 0;  // column shapes only: 4, 1, 3, each with the stored geometry where timed
   for (int ci = 1; ci < NMAX; ++ci)
     if (use[ci] && (cands[ci] == 1 || cands[ci] == 3 || cands[ci] == 4) && best[ci] < 0.97f * best[fc]) fc = ci;
@@ -1744,6 +1752,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
     }
     LevelDesc<double> d{};
     double *geo_l = nullptr, *geox_l = nullptr;
+    float *geop_l = nullptr;
     d.dim = dim;
     d.k = k;
     for (int a = 0; a < 3; ++a) {
@@ -1850,6 +1859,15 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
           SMF_CUDA_OK(cudaGetLastError());
         }
       }
+      // coefficients of the FP32 plane kernel (2,304 B a cell), the same budget
+      const char *np = getenv("STOKES_NO_PLANE");
+      const long long pbytes = pl_geometry_bytes(cells);
+      if (g64 && k == 2 && !C->det && !(np && np[0] == '1') && pbytes <= (long long)(total_b / 16) &&
+          pbytes <= (long long)(free_b / 4)) {
+        if ((st = dalloc(C, &geop_l, pbytes / (long long)sizeof(float)))) return st;
+        launch_pl_geometry(d, geop_l, C->s);
+        SMF_CUDA_OK(cudaGetLastError());
+      }
       // FP32 levels of at most 32^3 cells (56.6 MB for k = 2): stored as a candidate that the
       // setup's timing keeps or drops per level.  On the small levels a launch is a dependency
       // chain (vertex loads, Jacobian, adjugate and its division, then the contractions); stored
@@ -1866,6 +1884,11 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
     C->L32[l].d = f;
     C->L64[l].geo = geo_l;
     C->L64[l].geox = geox_l;
+    C->L32[l].geox = geop_l;
+    {
+      const char *np = getenv("STOKES_NO_PLANE");
+      C->L32[l].plane = dim == 3 && k == 2 && !C->det && !(np && np[0] == '1') && (!mesh->vertices || geop_l);
+    }
     if ((st = alloc_level_buffers(C, C->L64[l]))) return st;
     if ((st = alloc_level_buffers(C, C->L32[l]))) return st;
   }
@@ -3657,11 +3680,11 @@ int stokes_time_apply(stokes_ctx *C, int level, int precision, int blocks, int r
     if (precision == 64) {
       LevelRT<double> &R = C->L64[level];
       launch_cell_apply<double>(R.d, C->tab64, Runner<double>(C).form(blocks), R.x, R.x + R.d.n_u, R.r, R.r + R.d.n_u,
-                                C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr);
+                                C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr, R.plane);
     } else {
       LevelRT<float> &R = C->L32[level];
       launch_cell_apply<float>(R.d, C->tab32, Runner<float>(C).form(blocks), R.x, R.x + R.d.n_u, R.r, R.r + R.d.n_u,
-                               C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr);
+                               C->s, R.shape, R.geo, R.geox, R.rho, C->det ? &C->gb : nullptr, R.plane);
     }
     ++C->launches;
   }

@@ -32,8 +32,8 @@
 // operator's error is a third to a sixth of the FP64 column kernel's on random vectors and no larger on smooth ones
 // (tests/test_gpu_fixed_point.py).  One rounding to FP64 before the scatter.
 //
-// Measured (us, floating-point column kernel -> this kernel): 32^3 trilinear K 348 -> 92, A 264 -> 64, B^T 136 ->
-// 40, B 146 -> 32; 32^3 Cartesian K 401 -> 77, A 327 -> 51; 16^3 trilinear K 61 -> 18; 8^3 K 23 -> 11.  Bound by
+// Measured (us, floating-point column kernel -> this kernel): 32^3 trilinear K 348 -> 97, A 264 -> 62, B^T 136 ->
+// 36, B 146 -> 32; 32^3 Cartesian K 401 -> 80, A 327 -> 52; 16^3 trilinear K 61 -> 19; 8^3 K 23 -> 11.  Bound by
 // the instruction chains of 12 resident warps per SM (168 registers): issue 38 % busy, most stalls fixed latencies.
 //
 // Warps with a value that is not finite, or whose largest is outside 2^-850 .. 2^850, take the same
@@ -53,9 +53,11 @@ typedef long long i64;
 
 constexpr int kFxCells = 10;   // cells per warp
 constexpr int kFxThreads = 96;  // a CTA is the three components of one group of 10 cells
-constexpr int kFxFields = 16;  // stored per Gauss point: G 00 01 02 11 12 22, W, C (column c at 7 + 3 c)
-// int2 entries of a level's stored coefficients: [group of 10 cells][y, x point][field][lane], then two scales per cell
-__host__ __device__ inline long long fx_group_entries() { return 9ll * kFxFields * 32; }
+// Stored coefficients of a level, int2 entries: [group of 10 cells] times a block of G 00 01 02 11 12 22 and W and a
+// block of C (column c at 3 c), each [y, x point][field][lane], so that a launch copies what it needs of a group as one
+// or two contiguous pieces; then two scales per cell.
+constexpr int kFxG = 7, kFxC = 9;
+__host__ __device__ inline long long fx_group_entries() { return 9ll * (kFxG + kFxC) * 32; }
 __host__ __device__ inline long long fx_entries(long long cells) {
   return (cells + kFxCells - 1) / kFxCells * fx_group_entries() + cells;
 }
@@ -81,12 +83,16 @@ __device__ __forceinline__ i64 fx_wide_imm(int a, i64 c) {
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "n"(B), "l"(c));
   return r;
 }
+constexpr int kFxWUp = 3;    // W's digits stand for 2^-kFxWUp of its scale (FxInt::value_up)
+constexpr int kFxTDown = 3;  // integers: places the test sums are shifted down before the transposed interpolation
+
 template <int H, int L>
 struct FxTab {};  // the constant (H 2^32 + L) / 2^64
 
 struct FxInt {
   typedef i64 V;
   typedef Dig C;
+  static constexpr bool SPLIT = true;  // whole parts of table entries are added apart (entries stay below 1/2)
   static __device__ __forceinline__ C tab(int h, int l) { return {h, l}; }
   static __device__ __forceinline__ V zero() { return 0; }
   // base + sum of c v / 2^64, rounded to nearest: rounding down would add up over the cells (the product of
@@ -127,37 +133,41 @@ struct FxInt {
   static __device__ __forceinline__ V down(V v) {  // v / 2^N, halves to even
     return (v + ((1 << (N - 1)) - 1) + ((v >> N) & 1)) >> N;
   }
+  static __device__ __forceinline__ V half(V v) { return down<1>(v); }
+  static __device__ __forceinline__ V tdown(V v) { return down<kFxTDown>(v); }
   static __device__ __forceinline__ V down_by(V v, int n) { return v >> n; }  // n large: the lost part is below the other term's rounding
 };
-struct FxDbl {
-  typedef double V;
-  typedef double C;
-  static __device__ __forceinline__ C tab(int h, int l) { return h * 0x1p-32 + l * 0x1p-64; }
-  static __device__ __forceinline__ V zero() { return 0.0; }
+template <typename T>
+struct FxFloat {
+  typedef T V;
+  typedef T C;
+  static constexpr bool SPLIT = false;
+  static __device__ __forceinline__ C tab(int h, int l) { return (T)(h * 0x1p-32 + l * 0x1p-64); }
+  static __device__ __forceinline__ V zero() { return T(0); }
   struct Sum {
-    double s;
+    T s;
   };
   static __device__ __forceinline__ Sum start(V base, C c, V v) { return {base + c * v}; }
   static __device__ __forceinline__ void add(Sum &s, C c, V v) { s.s += c * v; }
   template <int H, int L>
   static __device__ __forceinline__ Sum start(V base, FxTab<H, L>, V v) {
-    return {base + (H * 0x1p-32 + L * 0x1p-64) * v};
+    return {base + (T)(H * 0x1p-32 + L * 0x1p-64) * v};
   }
   template <int H, int L>
   static __device__ __forceinline__ void add(Sum &s, FxTab<H, L>, V v) {
-    s.s += (H * 0x1p-32 + L * 0x1p-64) * v;
+    s.s += (T)(H * 0x1p-32 + L * 0x1p-64) * v;
   }
   static __device__ __forceinline__ V value(const Sum &s) { return s.s; }
   template <int N>
   static __device__ __forceinline__ V value_up(const Sum &s) {
     return s.s;
   }
-  template <int N>
-  static __device__ __forceinline__ V down(V v) {
-    return v * (1.0 / (1 << N));
-  }
+  static __device__ __forceinline__ V half(V v) { return T(0.5) * v; }
+  static __device__ __forceinline__ V tdown(V v) { return v; }
   static __device__ __forceinline__ V down_by(V v, int) { return v; }
 };
+typedef FxFloat<double> FxDbl;
+typedef FxFloat<float> FxFlt;
 // Table entries (times 2^64 as digits).
 using FxTS00M = FxTab<-1343043426, -896144430>;     // 0.3 + r - 1 (the unit part is the base of the sum)
 using FxTS01 = FxTab<1717986918, 1717986918>;    // 0.4
@@ -188,7 +198,7 @@ __device__ __forceinline__ void fx_interp_t(typename P::V &a, typename P::V &b, 
 // pressure: two node values -> three Gauss values, and the transpose
 template <typename P>
 __device__ __forceinline__ void fx_pre(typename P::V p0, typename P::V p1, typename P::V (&q)[3]) {
-  const typename P::V m = P::template down<1>(p0 + p1), d = P::value(P::start(P::zero(), FxTR{}, p0 - p1));
+  const typename P::V m = P::half(p0 + p1), d = P::value(P::start(P::zero(), FxTR{}, p0 - p1));
   q[0] = m + d;
   q[1] = m;
   q[2] = m - d;
@@ -196,7 +206,7 @@ __device__ __forceinline__ void fx_pre(typename P::V p0, typename P::V p1, typen
 template <typename P>
 __device__ __forceinline__ void fx_pre_t(typename P::V q0, typename P::V q1, typename P::V q2, typename P::V &p0,
                                          typename P::V &p1) {
-  const typename P::V e = P::template down<1>(q0 + q1 + q2), o = P::value(P::start(P::zero(), FxTR{}, q0 - q2));
+  const typename P::V e = P::half(q0 + q1 + q2), o = P::value(P::start(P::zero(), FxTR{}, q0 - q2));
   p0 = e + o;
   p1 = e - o;
 }
@@ -211,8 +221,6 @@ __host__ __device__ inline int fx_exp(double x) { return x > 0.0 ? ilogb(x) + 1 
 // Scales of a cell's coefficients: the x and y rows of G together, and its z row, sum to at most 2^62 in absolute
 // value (only x and y fluxes add up in a plane's test sums), W (stored 2^-kFxWUp of
 // its scale, FxInt::value_up) to 2^62; columns of C to 2^62.
-constexpr int kFxWUp = 3;
-constexpr int kFxTDown = 3;  // places the test sums are shifted down before the transposed interpolation
 __host__ __device__ inline int fx_scale_g(double xy, double z, double w) {
   const int a = fx_exp(xy > z ? xy : z) - 62, b = fx_exp(w) - 62 - kFxWUp;
   return a > b ? a : b;
@@ -271,34 +279,74 @@ template <typename P, bool CART>
 struct FxGeo;
 template <>
 struct FxGeo<FxInt, false> {
-  const int2 *g;  // shared memory: this lane's entry of field 0 at point 0, `fields` staged per point
-  int f0, fields;
+  const int2 *g, *cc;  // shared memory: this lane's first entries of the staged blocks
   __device__ __forceinline__ Dig at(int pt, int f) const {
-    const int2 v = g[(pt * fields + f - f0) * 32];
+    const int2 v = g[(pt * kFxG + f) * 32];
     return {v.x, v.y};
+  }
+  __device__ __forceinline__ Dig col(int pt, int c, int a) const {
+    const int2 v = cc[(pt * kFxC + 3 * c + a) * 32];
+    return {v.x, v.y};
+  }
+  template <int MODE>
+  __device__ __forceinline__ const FxGeo &point(int, int) const {
+    return *this;
   }
 };
 template <>
 struct FxGeo<FxDbl, false> {
-  const int2 *g;
-  int f0, fields;
+  FxGeo<FxInt, false> d;
   int eg, ec;
   __device__ __forceinline__ double at(int pt, int f) const {
-    const int2 v = g[(pt * fields + f - f0) * 32];
-    return fx_coef_value({v.x, v.y}, f < 6 ? eg : (f == 6 ? eg + kFxWUp : ec));
+    return fx_coef_value(d.at(pt, f), f < 6 ? eg : eg + kFxWUp);
+  }
+  __device__ __forceinline__ double col(int pt, int c, int a) const { return fx_coef_value(d.col(pt, c, a), ec); }
+  template <int MODE>
+  __device__ __forceinline__ const FxGeo &point(int, int) const {
+    return *this;
   }
 };
-// The staged fields of a launch: G and W with an A block, C with B or B^T.
+// FP32: quads of (G00, G01, G02, G11), (G12, G22, W, -) and a column of C per component, one point in registers.
+template <>
+struct FxGeo<FxFlt, false> {
+  const float4 *g, *cc;  // shared memory: this lane's first quads of the staged blocks
+  struct Point {
+    float4 a, b, d;
+    __device__ __forceinline__ float at(int, int i) const {
+      return i == 0 ? a.x : (i == 1 ? a.y : (i == 2 ? a.z : (i == 3 ? a.w : (i == 4 ? b.x : (i == 5 ? b.y : b.z)))));
+    }
+    __device__ __forceinline__ float col(int, int, int k) const { return k == 0 ? d.x : (k == 1 ? d.y : d.z); }
+  };
+  template <int MODE>
+  __device__ __forceinline__ Point point(int pt, int c) const {
+    Point q;
+    if (MODE & kApplyA) {
+      q.a = g[2 * pt * 32];
+      q.b = g[(2 * pt + 1) * 32];
+    }
+    if (MODE & (kApplyB | kApplyBT)) q.d = cc[(3 * pt + c) * 32];
+    return q;
+  }
+};
+// What a launch stages: the G block with an A block, the C block with B or B^T.
 template <int MODE>
 struct FxStage {
-  static constexpr int F0 = (MODE & kApplyA) ? 0 : 7;
-  static constexpr int FIELDS = ((MODE & (kApplyB | kApplyBT)) ? kFxFields : 7) - F0;
-  static constexpr int BYTES = 9 * FIELDS * 32 * (int)sizeof(int2);
+  static constexpr int G = (MODE & kApplyA) ? 9 * kFxG * 32 * (int)sizeof(int2) : 0;
+  static constexpr int C = (MODE & (kApplyB | kApplyBT)) ? 9 * kFxC * 32 * (int)sizeof(int2) : 0;
 };
 template <typename P>
 struct FxGeo<P, true> {
   typename P::C g[3][3], w[3], cc[3];  // [direction][weight class]
 };
+
+template <int MODE, typename P>
+__device__ __forceinline__ const FxGeo<P, true> &fx_point(const FxGeo<P, true> &g, int, int) {
+  return g;
+}
+template <int MODE, typename P>
+__device__ __forceinline__ decltype(auto) fx_point(const FxGeo<P, false> &g, int pt, int c) {
+  return g.template point<MODE>(pt, c);
+}
 
 // The element action on a thread's plane.  v: in the 9 node values of plane z (scaled integers, or
 // doubles), out the 9 test sums of that node plane times 2^-kFxTDown;
@@ -330,6 +378,12 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
     d0 = z == 0 ? e0 : (z == 1 ? o : ne0);
     d1 = z == 0 ? S01 : (z == 1 ? e3 : ne2);
     d2 = z == 0 ? e2 : (z == 1 ? ne3 : nS01);
+    if constexpr (!P::SPLIT) {  // the whole parts belong to the table
+      s0 += P::zero() + 1;
+      d0 += z == 0 ? -2 : (z == 1 ? 0 : 2);
+      d1 += z == 0 ? 2 : (z == 1 ? 1 : 0);
+      d2 += z == 0 ? 0 : (z == 1 ? -1 : -2);
+    }
   }
   V pq[3][3];
   if (DO_BT) {
@@ -340,7 +394,7 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
       V m[2];
 #pragma unroll
       for (int x = 0; x < 2; ++x)
-        m[x] = P::value(P::start(P::template down<1>(pr[0][y][x] + pr[1][y][x]), rz, pr[0][y][x] - pr[1][y][x]));
+        m[x] = P::value(P::start(P::half(pr[0][y][x] + pr[1][y][x]), rz, pr[0][y][x] - pr[1][y][x]));
       fx_pre<P>(m[0], m[1], t[y]);
     }
 #pragma unroll
@@ -362,8 +416,13 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
         const V a = v[y][x], b = __shfl_sync(FULL, a, l1), e = __shfl_sync(FULL, a, l2);
-        const V w = (z == 2 ? a : b) - (z == 0 ? a : e);
-        typename P::Sum q = P::start(a, s0, a), g = P::start(z == 1 ? w : 2 * w, d0, a);
+        V qb = P::zero(), gb = P::zero();
+        if constexpr (P::SPLIT) {
+          const V w = (z == 2 ? a : b) - (z == 0 ? a : e);
+          qb = a;
+          gb = z == 1 ? w : 2 * w;
+        }
+        typename P::Sum q = P::start(qb, s0, a), g = P::start(gb, d0, a);
         P::add(q, s1, b);
         P::add(g, d1, b);
         P::add(q, s2, e);
@@ -404,6 +463,7 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
       }
       const V gzp = NEED_U ? gz[y][x] : P::zero();
       V a0 = P::zero(), a1 = P::zero(), a2 = P::zero();
+      decltype(auto) pg = fx_point<MODE>(geo, pt, c);
       if constexpr (DO_A) {
         V w;
         if constexpr (CART) {
@@ -412,19 +472,19 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
           a2 = P::value(P::start(P::zero(), geo.g[2][m], gzp));
           w = P::template value_up<kFxWUp>(P::start(P::zero(), geo.w[m], v[y][x]));
         } else {
-          const Cf g1 = geo.at(pt, 1), g2 = geo.at(pt, 2), g4 = geo.at(pt, 4);
-          typename P::Sum q0 = P::start(P::zero(), geo.at(pt, 0), gx), q1 = P::start(P::zero(), g1, gx),
+          const Cf g1 = pg.at(pt, 1), g2 = pg.at(pt, 2), g4 = pg.at(pt, 4);
+          typename P::Sum q0 = P::start(P::zero(), pg.at(pt, 0), gx), q1 = P::start(P::zero(), g1, gx),
                           q2 = P::start(P::zero(), g2, gx);
           P::add(q0, g1, gy);
-          P::add(q1, geo.at(pt, 3), gy);
+          P::add(q1, pg.at(pt, 3), gy);
           P::add(q2, g4, gy);
           P::add(q0, g2, gzp);
           P::add(q1, g4, gzp);
-          P::add(q2, geo.at(pt, 5), gzp);
+          P::add(q2, pg.at(pt, 5), gzp);
           a0 = P::value(q0);
           a1 = P::value(q1);
           a2 = P::value(q2);
-          w = P::template value_up<kFxWUp>(P::start(P::zero(), geo.at(pt, 6), v[y][x]));
+          w = P::template value_up<kFxWUp>(P::start(P::zero(), pg.at(pt, 6), v[y][x]));
         }
         if (DO_BT) {
           a0 = P::down_by(a0, sa);
@@ -445,7 +505,7 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
           }
           if (DO_B) qa[y][x] = -P::value(P::start(P::zero(), k, c == 0 ? gx : (c == 1 ? gy : gzp)));
         } else {
-          const Cf c0 = geo.at(pt, 7 + 3 * c), c1 = geo.at(pt, 8 + 3 * c), c2 = geo.at(pt, 9 + 3 * c);
+          const Cf c0 = pg.col(pt, c, 0), c1 = pg.col(pt, c, 1), c2 = pg.col(pt, c, 2);
           if (DO_BT) {
             a0 -= P::value(P::start(P::zero(), c0, pq[y][x]));
             a1 -= P::value(P::start(P::zero(), c1, pq[y][x]));
@@ -490,10 +550,15 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
     for (int y = 0; y < 3; ++y)
 #pragma unroll
       for (int x = 0; x < 3; ++x) {
-        const V a = P::template down<kFxTDown>(t[y][x]), f = P::template down<kFxTDown>(gz[y][x]);
-        const V w = z == 1 ? f : 2 * f;
-        typename P::Sum c0 = P::start(a + (z == 0 ? -w : (z == 1 ? P::zero() : w)), s0, a),
-                        c1 = P::start(z == 2 ? P::zero() : w, s1, a), c2 = P::start(z == 0 ? P::zero() : -w, s2, a);
+        const V a = P::tdown(t[y][x]), f = P::tdown(gz[y][x]);
+        V b0 = P::zero(), b1 = P::zero(), b2 = P::zero();
+        if constexpr (P::SPLIT) {
+          const V w = z == 1 ? f : 2 * f;
+          b0 = a + (z == 0 ? -w : (z == 1 ? P::zero() : w));
+          b1 = z == 2 ? P::zero() : w;
+          b2 = z == 0 ? P::zero() : -w;
+        }
+        typename P::Sum c0 = P::start(b0, s0, a), c1 = P::start(b1, s1, a), c2 = P::start(b2, s2, a);
         P::add(c0, d0, f);
         P::add(c1, d1, f);
         P::add(c2, d2, f);
@@ -517,93 +582,111 @@ __device__ __forceinline__ void fx_plane(typename P::V (&v)[3][3], const typenam
       for (int x = 0; x < 2; ++x) {
         const V a = w[y][x], b = __shfl_sync(FULL, a, l1), e = __shfl_sync(FULL, a, l2);
         // plane 0: own - plane 2 (l2); plane 2: own - plane 0 (l1); both sums add r times that
-        qn[y][x] = P::value(P::start(P::template down<1>(a + b + e), FxTR{}, a - (z == 0 ? e : b)));
+        qn[y][x] = P::value(P::start(P::half(a + b + e), FxTR{}, a - (z == 0 ? e : b)));
       }
   }
 }
 
-// One warp's cells of one component.  FUSED: see Fuse and cc_group.
-template <int MODE, bool CART, bool FUSED>
-__device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const double *__restrict__ u,
-                                         const double *__restrict__ p, double *__restrict__ yu, double *__restrict__ yp,
-                                         const int2 *__restrict__ geo, long long group, int c, const FxCart &K, const Fuse<double> &F) {
-  constexpr bool DO_A = MODE & kApplyA, DO_BT = MODE & kApplyBT, DO_B = MODE & kApplyB;
-  constexpr bool NEED_U = DO_A || DO_B;
-  constexpr unsigned FULL = 0xffffffffu;
-  // Trilinear cells: the group's coefficients go to shared memory while the values are gathered (without it a warp waited for them at every point: 10.4 of 15 stall cycles an issue).
-  extern __shared__ int4 fx_smem[];
-  if constexpr (!CART) {
-    using ST = FxStage<MODE>;
-    constexpr int PER = ST::FIELDS * 16;  // 16-byte pieces a point
-    const int4 *src = reinterpret_cast<const int4 *>(geo + group * fx_group_entries() + ST::F0 * 32);
-    for (int i = threadIdx.x; i < 9 * PER; i += kFxThreads) {
-      const int pt = i / PER;
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(fx_smem + i);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src + i + pt * (kFxFields * 16 - PER)) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  const int lane = threadIdx.x & 31;
-  const bool pad = lane >= 30;
-  const int z = pad ? 0 : lane / 10, s = pad ? 0 : lane - 10 * z;
+// ---- a warp's cells of one component: indices, gathers, scatter (any precision) ---------------------------
+struct PlaneIdx {
+  int lane, z, cx, cy, cz;
+  bool fast;  // FP32: every node of the warp's cells is free, no per-node predicates (FP64's code is long enough)
+  bool pad, valid, fx[3], fy[3];
+  unsigned cell;
+  long long N0, P0, P01, vbase, pbase;
+};
+template <typename T>
+__device__ __forceinline__ PlaneIdx plane_index(const LevelDesc<T> &L, long long group, int c) {
+  PlaneIdx I;
+  I.lane = threadIdx.x & 31;
+  I.pad = I.lane >= 30;
+  I.z = I.pad ? 0 : I.lane / 10;
+  const int s = I.pad ? 0 : I.lane - 10 * I.z;
   const long long cell_raw = group * kFxCells + s;
-  const bool valid = !pad && cell_raw < L.n_cells;
-  const unsigned cell = (unsigned)(valid ? cell_raw : 0);  // launches hold n_cells below 2^31
-  const int cx = (int)(cell % (unsigned)L.n[0]);
-  const unsigned rr = cell / (unsigned)L.n[0];
-  const int cy = (int)(rr % (unsigned)L.n[1]), cz = (int)(rr / (unsigned)L.n[1]);
-  const int gx0 = 2 * cx, gy0 = 2 * cy, gz0 = 2 * cz + z;
-  bool fx[3], fy[3];
-  const bool fz = valid && !((L.faces & 16u) && gz0 == 0) && !((L.faces & 32u) && gz0 == L.N[2] - 1);
+  I.valid = !I.pad && cell_raw < L.n_cells;
+  I.cell = (unsigned)(I.valid ? cell_raw : 0);  // launches hold n_cells below 2^31
+  I.cx = (int)(I.cell % (unsigned)L.n[0]);
+  const unsigned rr = I.cell / (unsigned)L.n[0];
+  I.cy = (int)(rr % (unsigned)L.n[1]);
+  I.cz = (int)(rr / (unsigned)L.n[1]);
+  const int gx0 = 2 * I.cx, gy0 = 2 * I.cy, gz0 = 2 * I.cz + I.z;
+  const bool fz = I.valid && !((L.faces & 16u) && gz0 == 0) && !((L.faces & 32u) && gz0 == L.N[2] - 1);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    fx[i] = fz && !((L.faces & 1u) && gx0 + i == 0) && !((L.faces & 2u) && gx0 + i == L.N[0] - 1);
-    fy[i] = !((L.faces & 4u) && gy0 + i == 0) && !((L.faces & 8u) && gy0 + i == L.N[1] - 1);
+    I.fx[i] = fz && !((L.faces & 1u) && gx0 + i == 0) && !((L.faces & 2u) && gx0 + i == L.N[0] - 1);
+    I.fy[i] = !((L.faces & 4u) && gy0 + i == 0) && !((L.faces & 8u) && gy0 + i == L.N[1] - 1);
   }
-  const long long N0 = L.N[0];
-  const long long vbase = c * L.nv + ((long long)gz0 * L.N[1] + gy0) * N0 + gx0;
-  const long long P0 = L.Pn[0], P01 = (long long)L.Pn[0] * L.Pn[1];
-  const long long pbase = ((long long)cz * L.Pn[1] + cy) * P0 + cx;
-
-  double uv[3][3], pv[2][2][2];
+  I.fast = sizeof(T) == 4 && __all_sync(0xffffffffu, I.pad || (I.fx[0] && I.fx[1] && I.fx[2] && I.fy[0] && I.fy[1] && I.fy[2]));
+  I.N0 = L.N[0];
+  I.vbase = c * L.nv + ((long long)gz0 * L.N[1] + gy0) * I.N0 + gx0;
+  I.P0 = L.Pn[0];
+  I.P01 = (long long)L.Pn[0] * L.Pn[1];
+  I.pbase = ((long long)I.cz * L.Pn[1] + I.cy) * I.P0 + I.cx;
+  return I;
+}
+// The 9 node values of the thread's plane and the cell's 8 pressure values.  FUSED: the Fuse combinations, and
+// the owner of each node performs their side effects (see Fuse and cc_group).
+template <int MODE, bool FUSED, typename T>
+__device__ __forceinline__ void plane_gather(const LevelDesc<T> &L, const PlaneIdx &I, int c, const T *__restrict__ u,
+                                             const T *__restrict__ p, const Fuse<T> &F, T (&uv)[3][3], T (&pv)[2][2][2]) {
+  constexpr bool NEED_U = MODE & (kApplyA | kApplyB), DO_BT = MODE & kApplyBT;
   if constexpr (FUSED) {
-    const bool oz = valid && (z < 2 || cz == L.n[2] - 1);
+    const bool oz = I.valid && (I.z < 2 || I.cz == L.n[2] - 1);
     bool ox[3], oy[3];  // this cell owns the node (local index below the last, or last cell)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      ox[i] = oz && (i < 2 || cx == L.n[0] - 1);
-      oy[i] = i < 2 || cy == L.n[1] - 1;
+      ox[i] = oz && (i < 2 || I.cx == L.n[0] - 1);
+      oy[i] = i < 2 || I.cy == L.n[1] - 1;
     }
+    T raw[kFuseVel + 2][3][3];  // every load first
 #pragma unroll
     for (int iy = 0; iy < 3; ++iy)
 #pragma unroll
       for (int ix = 0; ix < 3; ++ix) {
-        const long long gi = vbase + iy * N0 + ix;
-        const bool fr = fx[ix] && fy[iy], own = ox[ix] && oy[iy];
-        double val = 0.0;
-        if ((fr && NEED_U) || (own && F.vstore)) {
-          if (F.nv > 0) {
-            double sum = F.vc[0] * F.vv[0][gi];
+        const long long gi = I.vbase + iy * I.N0 + ix;
+        const bool need = (NEED_U && I.fx[ix] && I.fy[iy]) || (ox[ix] && oy[iy] && F.vstore);
+        if (F.nv > 0) {
 #pragma unroll
-            for (int j = 1; j < kFuseVel; ++j)
-              if (j < F.nv) sum += F.vc[j] * F.vv[j][gi];
-            val = (F.vb ? F.vb[gi] : 0.0) + (F.vd ? F.vd[gi] : 1.0) * sum;
-          } else {
-            val = u[gi];
-          }
-        }
-        uv[iy][ix] = fr ? val : 0.0;
-        if (own) {
-          if (F.vstore) F.vstore[gi] = val;
-          if (F.vzero[0]) F.vzero[0][gi] = 0.0;
-          if (F.vzero[1]) F.vzero[1][gi] = 0.0;
+          for (int j = 0; j < kFuseVel; ++j) raw[j][iy][ix] = (need && j < F.nv) ? F.vv[j][gi] : T(0);
+          raw[kFuseVel][iy][ix] = (need && F.vd) ? F.vd[gi] : T(1);
+          raw[kFuseVel + 1][iy][ix] = (need && F.vb) ? F.vb[gi] : T(0);
+        } else {
+          raw[0][iy][ix] = need ? u[gi] : T(0);
         }
       }
-  } else if (NEED_U) {
 #pragma unroll
     for (int iy = 0; iy < 3; ++iy)
 #pragma unroll
-      for (int ix = 0; ix < 3; ++ix) uv[iy][ix] = (fx[ix] && fy[iy]) ? u[vbase + iy * N0 + ix] : 0.0;
+      for (int ix = 0; ix < 3; ++ix) {
+        const long long gi = I.vbase + iy * I.N0 + ix;
+        T val = raw[0][iy][ix];
+        if (F.nv > 0) {
+          T sum = F.vc[0] * raw[0][iy][ix];
+#pragma unroll
+          for (int j = 1; j < kFuseVel; ++j)
+            if (j < F.nv) sum += F.vc[j] * raw[j][iy][ix];
+          val = raw[kFuseVel + 1][iy][ix] + raw[kFuseVel][iy][ix] * sum;
+        }
+        uv[iy][ix] = (I.fx[ix] && I.fy[iy]) ? val : T(0);
+        if (ox[ix] && oy[iy]) {
+          if (F.vstore) F.vstore[gi] = val;
+          if (F.vzero[0]) F.vzero[0][gi] = T(0);
+          if (F.vzero[1]) F.vzero[1][gi] = T(0);
+        }
+      }
+  } else if (NEED_U) {
+    const T *ub = u + I.vbase;
+    if (I.fast) {
+#pragma unroll
+      for (int iy = 0; iy < 3; ++iy)
+#pragma unroll
+        for (int ix = 0; ix < 3; ++ix) uv[iy][ix] = ub[iy * I.N0 + ix];
+    } else {
+#pragma unroll
+      for (int iy = 0; iy < 3; ++iy)
+#pragma unroll
+        for (int ix = 0; ix < 3; ++ix) uv[iy][ix] = (I.fx[ix] && I.fy[iy]) ? ub[iy * I.N0 + ix] : T(0);
+    }
   }
   if (DO_BT) {
 #pragma unroll
@@ -612,11 +695,11 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
       for (int a2 = 0; a2 < 2; ++a2)
 #pragma unroll
         for (int a1 = 0; a1 < 2; ++a1) {
-          const long long gi = pbase + a3 * P01 + a2 * P0 + a1;
-          double val = 0.0;
-          if (valid) {
+          const long long gi = I.pbase + a3 * I.P01 + a2 * I.P0 + a1;
+          T val = T(0);
+          if (I.valid) {
             if (FUSED && F.np > 0) {
-              double sum = 0.0;
+              T sum = T(0);
 #pragma unroll
               for (int j = 0; j < kFusePre; ++j)
                 if (j < F.np) sum += F.pc[j] * F.pv[j][gi];
@@ -626,27 +709,96 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
             }
           }
           pv[a3][a2][a1] = val;
-          if constexpr (FUSED) {  // once per node: component 0, planes 0 and 2 for the two z nodes
-            if (valid && c == 0 && z == 2 * a3 && (a1 < 1 || cx == L.n[0] - 1) && (a2 < 1 || cy == L.n[1] - 1) &&
-                (a3 < 1 || cz == L.n[2] - 1)) {
-              if (F.pacc) F.pacc[gi] += val;
-#pragma unroll
-              for (int j = 0; j < kFusePre; ++j)
-                if (F.pzero[j]) F.pzero[j][gi] = 0.0;
-            }
-          }
         }
+    if constexpr (FUSED) {  // once per node: component 0, planes 0 and 2 for the two z nodes
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int a1 = i & 1, a2 = (i >> 1) & 1, a3 = i >> 2;
+        if (I.valid && c == 0 && I.z == 2 * a3 && (a1 < 1 || I.cx == L.n[0] - 1) && (a2 < 1 || I.cy == L.n[1] - 1) &&
+            (a3 < 1 || I.cz == L.n[2] - 1)) {
+          const long long gi = I.pbase + a3 * I.P01 + a2 * I.P0 + a1;
+          if (F.pacc) F.pacc[gi] += pv[a3][a2][a1];
+#pragma unroll
+          for (int j = 0; j < kFusePre; ++j)
+            if (F.pzero[j]) F.pzero[j][gi] = T(0);
+        }
+      }
+    }
   }
+}
+template <int MODE, typename T>
+__device__ __forceinline__ void plane_scatter(const PlaneIdx &I, T *__restrict__ yu, T *__restrict__ yp, const T (&yv)[3][3],
+                                              const T (&qv)[2][2]) {
+  if (MODE & (kApplyA | kApplyBT)) {
+    T *yb = yu + I.vbase;
+    if (I.fast) {
+      if (!I.pad) {
+#pragma unroll
+        for (int iy = 0; iy < 3; ++iy)
+#pragma unroll
+          for (int ix = 0; ix < 3; ++ix) atomicAdd(&yb[iy * I.N0 + ix], yv[iy][ix]);
+      }
+    } else {
+#pragma unroll
+      for (int iy = 0; iy < 3; ++iy)
+#pragma unroll
+        for (int ix = 0; ix < 3; ++ix)
+          if (I.fx[ix] && I.fy[iy]) atomicAdd(&yb[iy * I.N0 + ix], yv[iy][ix]);
+    }
+  }
+  if (MODE & kApplyB) {
+    if (I.valid && I.z != 1) {
+#pragma unroll
+      for (int iy = 0; iy < 2; ++iy)
+#pragma unroll
+        for (int ix = 0; ix < 2; ++ix) atomicAdd(&yp[I.pbase + (I.z >> 1) * I.P01 + iy * I.P0 + ix], qv[iy][ix]);
+    }
+  }
+}
+// A contiguous block to shared memory in 16-byte pieces, without waiting.
+template <int BYTES>
+__device__ __forceinline__ void plane_stage(const void *src, void *dst) {
+  const int4 *s = static_cast<const int4 *>(src) + threadIdx.x;
+  const unsigned d = (unsigned)__cvta_generic_to_shared(static_cast<int4 *>(dst) + threadIdx.x);
+  constexpr int N = BYTES / 16;
+#pragma unroll
+  for (int i = 0; i < (N + kFxThreads - 1) / kFxThreads; ++i)
+    if ((i + 1) * kFxThreads <= N || (int)threadIdx.x < N - i * kFxThreads)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + i * kFxThreads * 16), "l"(s + i * kFxThreads)
+                   : "memory");
+}
+
+// One warp's cells of one component in FP64.
+template <int MODE, bool CART, bool FUSED>
+__device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const double *__restrict__ u,
+                                         const double *__restrict__ p, double *__restrict__ yu, double *__restrict__ yp,
+                                         const int2 *__restrict__ geo, long long group, int c, const FxCart &K, const Fuse<double> &F) {
+  constexpr bool DO_A = MODE & kApplyA, DO_BT = MODE & kApplyBT, DO_B = MODE & kApplyB;
+  constexpr bool NEED_U = DO_A || DO_B;
+  constexpr unsigned FULL = 0xffffffffu;
+  // Trilinear cells: the group's coefficients go to shared memory while the values are gathered (without
+  // it a warp waited for them at every point: 10.4 of 15 stall cycles an issue).
+  extern __shared__ int4 fx_smem[];
+  using ST = FxStage<MODE>;
+  if constexpr (!CART) {
+    const int2 *src = geo + group * fx_group_entries();
+    plane_stage<ST::G>(src, fx_smem);
+    plane_stage<ST::C>(src + 9 * kFxG * 32, fx_smem + ST::G / 16);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  const PlaneIdx I = plane_index(L, group, c);
+  const int lane = I.lane, z = I.z;
+  const unsigned cell = I.cell;
+  double uv[3][3], pv[2][2][2];
+  plane_gather<MODE, FUSED>(L, I, c, u, p, F, uv, pv);
 
   // ---- coefficients and scales ---------------------------------------------------------------------
   int eg, ec;
-  const int2 *gp = nullptr;
   if constexpr (CART) {
     eg = K.eg;
     ec = K.ec;
     if (L.mu_cell && DO_A) eg = fx_scale_g(K.xy * L.mu_cell[cell], K.zz * L.mu_cell[cell], K.wtop);
   } else {
-    gp = reinterpret_cast<const int2 *>(fx_smem) + lane;
     const int2 e = __ldg(geo + (L.n_cells + kFxCells - 1) / kFxCells * fx_group_entries() + cell);
     eg = e.x;
     ec = e.y;
@@ -655,7 +807,7 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
   if (NEED_U) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) tu = max(tu, __double2hiint(uv[i / 3][i % 3]) & 0x7fffffff);
-    const int l1 = lane < 20 ? lane + 10 : (pad ? lane : lane - 20), l2 = lane < 10 ? lane + 20 : (pad ? lane : lane - 10);
+    const int l1 = lane < 20 ? lane + 10 : (I.pad ? lane : lane - 20), l2 = lane < 10 ? lane + 20 : (I.pad ? lane : lane - 10);
     tu = max(tu, max(__shfl_sync(FULL, tu, l1), __shfl_sync(FULL, tu, l2)));
   }
   if (DO_BT) {
@@ -720,9 +872,8 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
         }
       }
     } else {
-      g.g = gp;
-      g.f0 = FxStage<MODE>::F0;
-      g.fields = FxStage<MODE>::FIELDS;
+      g.g = reinterpret_cast<const int2 *>(fx_smem) + lane;
+      g.cc = reinterpret_cast<const int2 *>(fx_smem + ST::G / 16) + lane;
     }
     fx_plane<FxInt, MODE, CART>(v, pi, qn, g, c, z, lane, sa);
     const double kv = tu == 0 && tp == 0 ? 0.0 : fx_pow2(ev + kFxTDown), kq = tu == 0 ? 0.0 : fx_pow2(su + ec + 64);
@@ -747,41 +898,26 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
         g.cc[m] = K.cd[c] * w;
       }
     } else {
-      g.g = gp;
-      g.f0 = FxStage<MODE>::F0;
-      g.fields = FxStage<MODE>::FIELDS;
+      g.d.g = reinterpret_cast<const int2 *>(fx_smem) + lane;
+      g.d.cc = reinterpret_cast<const int2 *>(fx_smem + ST::G / 16) + lane;
       g.eg = eg;
       g.ec = ec;
     }
     double qn[2][2];
     fx_plane<FxDbl, MODE, CART>(uv, pv, qn, g, c, z, lane, 0);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) yv[i / 3][i % 3] = (double)(1 << kFxTDown) * uv[i / 3][i % 3];
+    for (int i = 0; i < 9; ++i) yv[i / 3][i % 3] = uv[i / 3][i % 3];
 #pragma unroll
     for (int i = 0; i < 4; ++i) qv[i >> 1][i & 1] = qn[i >> 1][i & 1];
   }
 
-  if (DO_A || DO_BT) {
-#pragma unroll
-    for (int iy = 0; iy < 3; ++iy)
-#pragma unroll
-      for (int ix = 0; ix < 3; ++ix)
-        if (fx[ix] && fy[iy]) atomicAdd(&yu[vbase + iy * N0 + ix], yv[iy][ix]);
-  }
-  if (DO_B) {
-    if (valid && z != 1) {
-#pragma unroll
-      for (int iy = 0; iy < 2; ++iy)
-#pragma unroll
-        for (int ix = 0; ix < 2; ++ix) atomicAdd(&yp[pbase + (z >> 1) * P01 + iy * P0 + ix], qv[iy][ix]);
-    }
-  }
+  plane_scatter<MODE>(I, yu, yp, yv, qv);
 }
 
 template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads, 4)
     stokes_cell_apply_fx(const LevelDesc<double> L, const double *__restrict__ u, const double *__restrict__ p,
-                         double *__restrict__ yu, double *__restrict__ yp, const int2 *__restrict__ geo, const FxCart K) {
+                         double *__restrict__ yu, double *__restrict__ yp, const int2 *__restrict__ geo, const __grid_constant__ FxCart K) {
   pdl_enter();
   fx_group<MODE, CART, false>(L, u, p, yu, yp, geo, blockIdx.x, threadIdx.x >> 5, K, Fuse<double>{});
 }
@@ -789,7 +925,7 @@ template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads, 4)
     stokes_cell_apply_fx_fused(const LevelDesc<double> L, const double *__restrict__ u, const double *__restrict__ p,
                                double *__restrict__ yu, double *__restrict__ yp, const int2 *__restrict__ geo,
-                               const FxCart K, const Fuse<double> F) {
+                               const __grid_constant__ FxCart K, const Fuse<double> F) {
   pdl_enter();
   fx_group<MODE, CART, true>(L, u, p, yu, yp, geo, blockIdx.x, threadIdx.x >> 5, K, F);
 }
@@ -864,7 +1000,7 @@ __global__ void k_fx_geometry(const LevelDesc<double> L, int2 *__restrict__ out)
     const Dd det = J[0][0] * adj[0][0] + J[1][0] * adj[0][1] + J[2][0] * adj[0][2];
     const Dd mu = {L.mu_cell ? L.mu_cell[cell] : L.mu, 0.0};
     const Dd wd = dd_div(A2 * mu * w, det);
-    Dd f[kFxFields];
+    Dd f[kFxG + kFxC];
     {
       auto dot = [&](int i, int j) { return wd * (adj[i][0] * adj[j][0] + adj[i][1] * adj[j][1] + adj[i][2] * adj[j][2]); };
       f[0] = dot(0, 0);
@@ -894,12 +1030,12 @@ __global__ void k_fx_geometry(const LevelDesc<double> L, int2 *__restrict__ out)
     }
     const int eg = fx_scale_g(xy, zz, wm), ec = fx_scale_c(cols);
     if (lane < 27) {
-      int2 *q = out + (cell / kFxCells) * fx_group_entries() + (lane % 9) * (kFxFields * 32) + iz * 10 + cell % kFxCells;
+      int2 *q = out + (cell / kFxCells) * fx_group_entries() + iz * 10 + cell % kFxCells;
 #pragma unroll
-      for (int i = 0; i < kFxFields; ++i) {
+      for (int i = 0; i < kFxG + kFxC; ++i) {
         const double s = ldexp(1.0, -(i < 6 ? eg : (i == 6 ? eg + kFxWUp : ec)));
         const Dig d = fx_split(__double2ll_rn(f[i].h * s) + __double2ll_rn(f[i].l * s));
-        q[i * 32] = make_int2(d.h, d.l);
+        q[(i < kFxG ? (lane % 9) * kFxG + i : 9 * kFxG + (lane % 9) * kFxC + (i - kFxG)) * 32] = make_int2(d.h, d.l);
       }
     }
     if (lane == 0) scales[cell] = make_int2(eg, ec);
@@ -917,12 +1053,12 @@ int launch_fx_mode(const LevelDesc<double> &L, const double *u, const double *p,
     if (L.cartesian)
       launch_kernel(stokes_cell_apply_fx_fused<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K, *F);
     else
-      launch_kernel(stokes_cell_apply_fx_fused<MODE, false>, grid, block, FxStage<MODE>::BYTES, s, L, u, p, yu, yp, g, K, *F);
+      launch_kernel(stokes_cell_apply_fx_fused<MODE, false>, grid, block, FxStage<MODE>::G + FxStage<MODE>::C, s, L, u, p, yu, yp, g, K, *F);
   } else {
     if (L.cartesian)
       launch_kernel(stokes_cell_apply_fx<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K);
     else
-      launch_kernel(stokes_cell_apply_fx<MODE, false>, grid, block, FxStage<MODE>::BYTES, s, L, u, p, yu, yp, g, K);
+      launch_kernel(stokes_cell_apply_fx<MODE, false>, grid, block, FxStage<MODE>::G + FxStage<MODE>::C, s, L, u, p, yu, yp, g, K);
   }
   return 0;
 }

@@ -15,7 +15,7 @@ double tridiag_max_eig(const std::vector<double> &a, const std::vector<double> &
 template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
                       cudaStream_t s, int shape, const T *geo = nullptr, const T *geox = nullptr, const T *rho = nullptr,
-                      const GridBarrier *det = nullptr);
+                      const GridBarrier *det = nullptr, bool plane = false);
 // `cols` vectors at once, ld entries apart (FP32)
 template <int K, typename T>
 int launch_cell_apply_cols_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
@@ -60,6 +60,11 @@ int launch_cell_apply_fx(const LevelDesc<double> &L, int mode, const double *u, 
                          const void *geo, const Fuse<double> *F, cudaStream_t s);
 long long fx_geometry_bytes(long long cells);
 void launch_fx_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
+// The FP32 kernel with a z plane per thread (shape 5 with LevelRT::plane, k = 2): as launch_cell_apply_fx.
+int launch_cell_apply_pl(const LevelDesc<float> &L, int mode, const float *u, const float *p, float *yu, float *yp,
+                         const void *geo, const Fuse<float> *F, cudaStream_t s);
+long long pl_geometry_bytes(long long cells);
+void launch_pl_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
 template <int K, typename T>
 int launch_cell_apply_cc_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp, const T *geo,
                            const GridBarrier *det, cudaStream_t s);
