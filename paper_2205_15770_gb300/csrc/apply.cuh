@@ -183,10 +183,10 @@ __global__ void __launch_bounds__(CellShape<DIM, K>::THREADS)
 
   int cx = 0, cy = 0, cz = 0;
   if (valid) {
-    cx = (int)(cell % L.n[0]);
-    long long r = cell / L.n[0];
-    cy = (int)(r % L.n[1]);
-    cz = (int)(r / L.n[1]);
+    cx = (int)((unsigned)cell % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+    const unsigned r = (unsigned)cell / (unsigned)L.n[0];
+    cy = (int)(r % (unsigned)L.n[1]);
+    cz = (int)(r / (unsigned)L.n[1]);
   }
   load_tables(tab, sm);
   if (!CART && t < CS::NVERT * DIM) {
@@ -593,10 +593,10 @@ __global__ void __launch_bounds__(CellShape<DIM, K>::THREADS)
   T *verts = bufA + CS::BUFS * NP;
   int cx = 0, cy = 0, cz = 0;
   if (valid) {
-    cx = (int)(cell % L.n[0]);
-    const long long r = cell / L.n[0];
-    cy = (int)(r % L.n[1]);
-    cz = (int)(r / L.n[1]);
+    cx = (int)((unsigned)cell % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+    const unsigned r = (unsigned)cell / (unsigned)L.n[0];
+    cy = (int)(r % (unsigned)L.n[1]);
+    cz = (int)(r / (unsigned)L.n[1]);
   }
   load_tables(tab, sm);
   if (!CART && t < CS::NVERT * DIM) {

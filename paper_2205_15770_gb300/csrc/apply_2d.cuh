@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(64)
   const int c = threadIdx.x >> 5;
   const long long cell = (long long)blockIdx.x * 32 + (threadIdx.x & 31);
   if (cell >= L.n_cells) return;
-  const int cx = (int)(cell % L.n[0]), cy = (int)(cell / L.n[0]);
+  const int cy = (int)((unsigned)cell / (unsigned)L.n[0]), cx = (int)((unsigned)cell - (unsigned)cy * (unsigned)L.n[0]);
   bool fx[N], fy[N];
 #pragma unroll
   for (int i = 0; i < N; ++i) {

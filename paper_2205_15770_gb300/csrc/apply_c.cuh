@@ -111,9 +111,9 @@ __device__ __forceinline__ long long pressure_node(const LevelDesc<T> &L, int cx
 
 template <int DIM, typename T>
 __device__ __forceinline__ void cell_coords(const LevelDesc<T> &L, long long cell, int &cx, int &cy, int &cz) {
-  cx = (int)(cell % L.n[0]);
-  const long long r = cell / L.n[0];
-  cy = (int)(r % L.n[1]);
+  cx = (int)((unsigned)cell % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+  const unsigned r = (unsigned)cell / (unsigned)L.n[0];
+  cy = (int)(r % (unsigned)L.n[1]);
   cz = DIM == 3 ? (int)(r / L.n[1]) : 0;
 }
 

@@ -232,10 +232,10 @@ __device__ __forceinline__ void cc_group(const LevelDesc<T> &L, const T *__restr
     const long long cell_raw = group * CPW + s;
     valid = !pad && cell_raw < L.n_cells;
     const long long cl = valid ? cell_raw : 0;
-    cx = (int)(cl % L.n[0]);
-    const long long rr = cl / L.n[0];
-    cy = (int)(rr % L.n[1]);
-    cz = (int)(rr / L.n[1]);
+    cx = (int)((unsigned)cl % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+    const unsigned rr = (unsigned)cl / (unsigned)L.n[0];
+    cy = (int)(rr % (unsigned)L.n[1]);
+    cz = (int)(rr / (unsigned)L.n[1]);
   } else {
     const long long ex = colour_extent(L.n, colour, 0), ey = colour_extent(L.n, colour, 1);
     const long long ez = colour_extent(L.n, colour, 2);

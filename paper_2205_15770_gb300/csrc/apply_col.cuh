@@ -213,10 +213,10 @@ __global__ void __launch_bounds__(32 * WARPS)
   const bool valid = !pad && cell < L.n_cells;
   int cx = 0, cy = 0, cz = 0;
   if (valid) {
-    cx = (int)(cell % L.n[0]);
-    const long long r = cell / L.n[0];
-    cy = (int)(r % L.n[1]);
-    cz = (int)(r / L.n[1]);
+    cx = (int)((unsigned)cell % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+    const unsigned r = (unsigned)cell / (unsigned)L.n[0];
+    cy = (int)(r % (unsigned)L.n[1]);
+    cz = (int)(r / (unsigned)L.n[1]);
   }
   auto lane_of = [&](int a, int b) { return base + b * NV + a; };
   // ownership of the gathered nodes (each node has exactly one owning cell)
@@ -676,9 +676,9 @@ __global__ void k_col_geometry(const LevelDesc<T> L, T *__restrict__ geo) {
   SMF_GRID_LOOP(t, L.n_cells * NV * NV) {
     const long long cell = t / (NV * NV);
     const int r = (int)(t - cell * NV * NV), iy = r / NV, ix = r - iy * NV;
-    const int cx = (int)(cell % L.n[0]);
-    const long long rr = cell / L.n[0];
-    const int cy = (int)(rr % L.n[1]), cz = (int)(rr / L.n[1]);
+    const int cx = (int)((unsigned)cell % (unsigned)L.n[0]);  // levels hold fewer than 2^31 cells
+    const unsigned rr = (unsigned)cell / (unsigned)L.n[0];
+    const int cy = (int)(rr % (unsigned)L.n[1]), cz = (int)(rr / (unsigned)L.n[1]);
     T G[NQ][6], Cm[NQ][9], Wd[NQ];
     const T mu = L.mu_cell ? L.mu_cell[cell] : L.mu;
     col_geometry<K, T, false, true>(L, ix, iy, cx, cy, cz, mu, L.gamma_rho, G, Cm, Wd);

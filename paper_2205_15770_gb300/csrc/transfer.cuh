@@ -32,6 +32,19 @@ struct XferTabs {
   int W = 0;
 };
 
+// Lattice node of DoF i of a level and its velocity component: compares and two 32-bit divisions (a space has
+// less than 2^31 nodes, see for_rows) where three 64-bit ones with their remainders took most of a transfer's time.
+template <typename T>
+__device__ __forceinline__ int xfer_node(long long i, bool vel, const LevelDesc<T> &L, const int *N, int &g0, int &g1, int &g2) {
+  const int c = vel ? (i >= L.nv) + (i >= 2 * L.nv) : 0;
+  const unsigned j = (unsigned)(vel ? i - c * L.nv : i - L.n_u), n0 = (unsigned)N[0], n1 = (unsigned)N[1];
+  const unsigned r = j / n0;
+  g0 = (int)(j - r * n0);
+  g2 = (int)(r / n1);
+  g1 = (int)(r - (unsigned)g2 * n1);
+  return c;
+}
+
 // Restriction row of coarse DoF i (P^T in, or P^T (in - minus) with SUB), summed over its (z, y)
 // term pairs t = t0, t0 + dt, ... (all of them for t0 = 0, dt = 1).
 template <typename T, int W, bool SUB, bool COH = false>
@@ -40,9 +53,9 @@ __device__ __forceinline__ T restrict_terms(const LevelDesc<T> &F, const LevelDe
   const bool vel = i < C.n_u;
   const int sp = vel ? 0 : 1;
   const int *Nc = vel ? C.N : C.Pn, *Nf = vel ? F.N : F.Pn;
-  const long long j = vel ? i % C.nv : i - C.n_u;
-  const int G0 = (int)(j % Nc[0]), G1 = (int)((j / Nc[0]) % Nc[1]), G2 = (int)(j / ((long long)Nc[0] * Nc[1]));
-  const long long off = vel ? (i / C.nv) * F.nv : F.n_u;
+  int G0, G1, G2;
+  const int comp = xfer_node(i, vel, C, Nc, G0, G1, G2);
+  const long long off = vel ? comp * F.nv : F.n_u;
   const T *src = in + off;
   const T *ssrc = SUB ? minus + off : nullptr;
   const Xfer1D<T> &ax = X.r[sp][0], &ay = X.r[sp][1], &az = X.r[sp][2];
@@ -55,8 +68,11 @@ __device__ __forceinline__ T restrict_terms(const LevelDesc<T> &F, const LevelDe
     w0[a] = a < n0 ? ax.w[G0 * W + a] : T(0);
   }
   T s = T(0);
-  for (int t = t0; t < n1 * n2; t += dt) {
-    const int a1 = t % n1, a2 = t / n1;
+  for (int t = t0, a2 = t0 / n1, a1 = t0 - a2 * n1; t < n1 * n2; t += dt, a1 += dt) {
+    while (a1 >= n1) {
+      a1 -= n1;
+      ++a2;
+    }
     const int f1 = ay.idx[G1 * W + a1], f2 = az.idx[G2 * W + a2];
     const T w21 = ay.w[G1 * W + a1] * az.w[G2 * W + a2];
     const long long ro = ((long long)f2 * Nf[1] + f1) * Nf[0];
@@ -115,9 +131,9 @@ __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDes
   const bool vel = i < F.n_u;
   const int sp = vel ? 0 : 1;
   const int *Nc = vel ? C.N : C.Pn, *Nf = vel ? F.N : F.Pn;
-  const long long j = vel ? i % F.nv : i - F.n_u;
-  const int g0 = (int)(j % Nf[0]), g1 = (int)((j / Nf[0]) % Nf[1]), g2 = (int)(j / ((long long)Nf[0] * Nf[1]));
-  const T *src = in + (vel ? (i / F.nv) * C.nv : C.n_u);
+  int g0, g1, g2;
+  const int comp = xfer_node(i, vel, F, Nf, g0, g1, g2);
+  const T *src = in + (vel ? comp * C.nv : C.n_u);
   const Xfer1D<T> &ax = X.p[sp][0], &ay = X.p[sp][1], &az = X.p[sp][2];
   const int n0 = ax.cnt[g0], n1 = ay.cnt[g1], n2 = az.cnt[g2];
   T s = T(0);
