@@ -549,10 +549,10 @@ struct Runner {
       tb = R.ps;
     }
     if (kd == 0) {
-      cheb_init_op(l, n, a, b, sr, Dinv, (T)cc.c0, (T *)nullptr, db, xb, base, scale, out, acc, za, zb);
+      cheb_init_op(l, n, a, b, sr, Dinv, (T)cc.c0, (T *)nullptr, (T *)nullptr, (T *)nullptr, base, scale, out, acc, za, zb);
       return;
     }
-    cheb_init_op(l, n, a, b, sr, Dinv, (T)cc.c0, rb, db, xb, (const T *)nullptr, T(0), (T *)nullptr, (T *)nullptr, za,
+    cheb_init_op(l, n, a, b, sr, Dinv, (T)cc.c0, rb, (T *)nullptr, xb, (const T *)nullptr, T(0), (T *)nullptr, (T *)nullptr, za,
                  zb);
     for (int j = 1; j <= kd; ++j) {
       if (velocity)
@@ -562,7 +562,8 @@ struct Runner {
       const bool last = j == kd;
       const T *bs = last ? base : nullptr;
       T *fo = last ? out : nullptr, *ac = last ? acc : nullptr;
-      cheb_step_op(l, n, rb, tb, Dinv, (T)cc.c1[j], (T)cc.c2[j], db, xb, bs, scale, fo, ac);
+      cheb_step_op(l, n, rb, tb, Dinv, (T)cc.c1[j], (T)cc.c2[j], db, xb, bs, scale, fo, ac,
+                   (j == 1 ? kChebFirst : 0) | (last ? kChebLast : 0));
     }
   }
   // The two Chebyshev vector kernels (k_cheb_init / k_cheb_step), launched or recorded.
@@ -586,10 +587,11 @@ struct Runner {
          sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb, n, ld);
   }
   void cheb_step_op(int l, long long n, const T *r, T *t, const T *Dinv, T c1, T c2, T *d, T *x, const T *base,
-                    T fscale, T *final_out, T *acc_out) {
+                    T fscale, T *final_out, T *acc_out, int flags) {
     if (rec()) {
       PqOp &o = rec_op(kPqChebStep, l);
       o.n = n;
+      o.add = flags;
       o.in[0] = fp(r);
       o.in[1] = fp(Dinv);
       o.in[2] = fp(base);
@@ -603,7 +605,7 @@ struct Runner {
       return;
     }
     vecp(k_cheb_step<T, 1>, k_cheb_step<T, VW>, {r, t, Dinv, d, x, base, final_out, acc_out}, n, r, t, Dinv, c1, c2,
-         d, x, base, fscale, final_out, acc_out, n, ld);
+         d, x, base, fscale, final_out, acc_out, flags, n, ld);
   }
   // y = B A^-1_hat B^T q   (y zero on entry)
   void S_tilde(int l, const T *q, T *y) {

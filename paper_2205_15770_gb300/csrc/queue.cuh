@@ -61,7 +61,7 @@ __device__ __forceinline__ void pq_item(const PqOp &o, long long b) {
                                             o.out[2], o.in[3], o.sc[2], o.out[3], o.out[4], o.out[5], o.out[6]);
           else
             cheb_step_packj<float, 4, true>(j, o.in[0], o.out[0], o.in[1], o.sc[0], o.sc[1], o.out[1], o.out[2],
-                                            o.in[2], o.sc[2], o.out[3], o.out[4]);
+                                            o.in[2], o.sc[2], o.out[3], o.out[4], o.add);
         }
         s0 = np4 * 4;
         if (b != o.items - 1) s1 = s0;  // the tail belongs to the last item
@@ -72,7 +72,7 @@ __device__ __forceinline__ void pq_item(const PqOp &o, long long b) {
                                       o.in[3], o.sc[2], o.out[3], o.out[4], o.out[5], o.out[6]);
         else
           cheb_step_elem<float, true>(i, o.in[0], o.out[0], o.in[1], o.sc[0], o.sc[1], o.out[1], o.out[2], o.in[2],
-                                      o.sc[2], o.out[3], o.out[4]);
+                                      o.sc[2], o.out[3], o.out[4], o.add);
       }
       break;
     }

@@ -38,7 +38,7 @@ struct PqOp {
   const float *in[4] = {};
   float *out[7] = {};
   float sc[3] = {};
-  int add = 0, n0 = 0;
+  int add = 0, n0 = 0;  // add: prolongation adds; a Chebyshev step's flags
   int vec4 = 0;  // Chebyshev steps: every vector 16-byte aligned (packs of 4)
   const double *Kinv = nullptr;
 };

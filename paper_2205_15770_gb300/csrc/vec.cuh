@@ -123,6 +123,7 @@ __device__ __forceinline__ Pack<T, V> ldpc_or0(const T *p, long long j) {
 // d = x = c0 * Dinv * r; r is stored if r_out != null.  za / zb (may alias a / b) are zeroed
 // after they are read: apply targets are kept zero between uses, so the cycle needs no memset.
 // With final_out / acc_out the degree-0 result f = base + fscale * x is written / accumulated.
+constexpr int kChebFirst = 1, kChebLast = 2;
 // One element of k_cheb_init / k_cheb_step (the scalar tail of the packed kernels, and the work
 // items of the persistent queue kernel with COH loads).
 template <typename T, bool COH = false>
@@ -135,21 +136,24 @@ __device__ __forceinline__ void cheb_init_elem(long long i, const T *a, const T 
   const T r = sr * (av - bv);
   if (r_out) r_out[i] = r;
   const T v = c0 * ld_in<COH>(Dinv + i) * r;
-  d[i] = v;
-  x[i] = v;
+  if (d) d[i] = v;
+  if (x) x[i] = v;
   const T f = (base ? ld_in<COH>(base + i) : T(0)) + fscale * v;
   if (final_out) final_out[i] = f;
   if (acc_out) acc_out[i] = ld_in<COH>(acc_out + i) + f;
 }
 template <typename T, bool COH = false>
 __device__ __forceinline__ void cheb_step_elem(long long i, const T *r, T *t, const T *Dinv, T c1, T c2, T *d, T *x,
-                                               const T *base, T fscale, T *final_out, T *acc_out) {
+                                               const T *base, T fscale, T *final_out, T *acc_out, int flags) {
   const T tv = ld_in<COH>(t + i);
   t[i] = T(0);
-  const T dn = c1 * ld_in<COH>(d + i) + c2 * ld_in<COH>(Dinv + i) * (ld_in<COH>(r + i) - tv);
-  const T xn = ld_in<COH>(x + i) + dn;
-  d[i] = dn;
-  x[i] = xn;
+  const T xv = ld_in<COH>(x + i);
+  const T dn = c1 * ((flags & kChebFirst) ? xv : ld_in<COH>(d + i)) + c2 * ld_in<COH>(Dinv + i) * (ld_in<COH>(r + i) - tv);
+  const T xn = xv + dn;
+  if (!(flags & kChebLast)) {
+    d[i] = dn;
+    x[i] = xn;
+  }
   const T f = (base ? ld_in<COH>(base + i) : T(0)) + fscale * xn;
   if (final_out) final_out[i] = f;
   if (acc_out) acc_out[i] = ld_in<COH>(acc_out + i) + f;
@@ -178,8 +182,8 @@ __device__ __forceinline__ void cheb_init_packj(long long j, const T *a, const T
     if (za) stp<V>(za, j, Z);
     if (zb) stp<V>(zb, j, Z);
     if (r_out) stp<V>(r_out, j, R);
-    stp<V>(d, j, X);
-    stp<V>(x, j, X);
+    if (d) stp<V>(d, j, X);
+    if (x) stp<V>(x, j, X);
     if (final_out || acc_out) {
       Pack<T, V> F, Anew;
 #pragma unroll
@@ -215,14 +219,18 @@ __global__ void k_cheb_init(const T *a, const T *b, T sr, const T *__restrict__ 
   SMF_TAIL_LOOP(i, n, V) cheb_init_elem(i, a, b, sr, Dinv, c0, r_out, d, x, base, fscale, final_out, acc_out, za, zb);
 }
 
-// One Chebyshev step: d = c1 d + c2 Dinv (r - t); x += d; t is zeroed after it is read.  With
+// One Chebyshev step: d = c1 d + c2 Dinv (r - t); x += d; t is zeroed after it is read.  kChebFirst: d equals x
+// on entry (the start stores it once); kChebLast: d and x are not needed any more.  With one step (k_A = 1) a pass
+// reads 4-5 and writes 2 vectors instead of 5-6 and 4, the start writes one less (32^3 FP32 cycle 946 -> 930 us).  With
 // final_out / acc_out, f = base + fscale * x_new is written / accumulated.
 template <typename T, int V, bool COH = false>
 __device__ __forceinline__ void cheb_step_packj(long long j, const T *r, T *t, const T *Dinv, T c1, T c2, T *d, T *x,
-                                                const T *base, T fscale, T *final_out, T *acc_out) {
+                                                const T *base, T fscale, T *final_out, T *acc_out, int flags) {
   {
     const Pack<T, V> R = ldpc<V, COH>(r, j), Tt = ldpc<V, COH>(t, j), Di = ldpc<V, COH>(Dinv, j),
-                     Dd = ldpc<V, COH>(d, j), X = ldpc<V, COH>(x, j);
+                     X = ldpc<V, COH>(x, j);
+    Pack<T, V> Dd = X;
+    if (!(flags & kChebFirst)) Dd = ldpc<V, COH>(d, j);
     const Pack<T, V> Bs = ldpc_or0<V, COH>(base, j), Ac = ldpc_or0<V, COH>(acc_out, j);
     Pack<T, V> Dn, Xn, Z;
 #pragma unroll
@@ -232,8 +240,10 @@ __device__ __forceinline__ void cheb_step_packj(long long j, const T *r, T *t, c
       Z.v[k] = T(0);
     }
     stp<V>(t, j, Z);
-    stp<V>(d, j, Dn);
-    stp<V>(x, j, Xn);
+    if (!(flags & kChebLast)) {
+      stp<V>(d, j, Dn);
+      stp<V>(x, j, Xn);
+    }
     if (final_out || acc_out) {
       Pack<T, V> F, Anew;
 #pragma unroll
@@ -249,7 +259,7 @@ __device__ __forceinline__ void cheb_step_packj(long long j, const T *r, T *t, c
 template <typename T, int V>
 __global__ void k_cheb_step(const T *__restrict__ r, T *__restrict__ t, const T *__restrict__ Dinv, T c1, T c2,
                             T *__restrict__ d, T *__restrict__ x, const T *__restrict__ base, T fscale,
-                            T *__restrict__ final_out, T *__restrict__ acc_out, long long n, long long ld) {
+                            T *__restrict__ final_out, T *__restrict__ acc_out, int flags, long long n, long long ld) {
   pdl_enter();
   r = column(r, ld);
   t = column(t, ld);
@@ -258,8 +268,8 @@ __global__ void k_cheb_step(const T *__restrict__ r, T *__restrict__ t, const T 
   base = column(base, ld);
   final_out = column(final_out, ld);
   acc_out = column(acc_out, ld);
-  SMF_PACK_LOOP(j, n, V) cheb_step_packj<T, V>(j, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out);
-  SMF_TAIL_LOOP(i, n, V) cheb_step_elem(i, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out);
+  SMF_PACK_LOOP(j, n, V) cheb_step_packj<T, V>(j, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out, flags);
+  SMF_TAIL_LOOP(i, n, V) cheb_step_elem(i, r, t, Dinv, c1, c2, d, x, base, fscale, final_out, acc_out, flags);
 }
 
 // End of a fused smoothing sequence: the last line of the compact Uzawa step,
