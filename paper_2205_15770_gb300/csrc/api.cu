@@ -303,6 +303,7 @@ struct stokes_ctx {
   double *Kinv = nullptr;
   // Krylov / Lanczos work space (FP64, finest level size)
   double *V = nullptr, *Z = nullptr, *w = nullptr, *hdev = nullptr, *partial = nullptr, *scal = nullptr;
+  double *lzs = nullptr;  // Lanczos coefficients (setup)
   double *lz0 = nullptr, *lz1 = nullptr, *lz2 = nullptr, *lz3 = nullptr, *sq = nullptr;
   int restart = 30;
   std::vector<void *> allocs;
@@ -1044,6 +1045,29 @@ __global__ void k_probe_vel(const LevelDesc<double> L, int comp, int P, int cx, 
     v[i] = on ? sqrt(DAinv[i]) : 0.0;
   }
 }
+// The same for colours c0 + blockIdx.y = (cz P + cy) P + cx, columns ld entries apart.
+__global__ void k_probe_vel_cols(const LevelDesc<double> L, int comp, int P, int c0, const double *__restrict__ DAinv,
+                                 double *__restrict__ v, long long ld) {
+  const int col = c0 + (int)blockIdx.y, cx = col % P, cy = (col / P) % P, cz = col / (P * P);
+  double *vc = v + blockIdx.y * ld;
+  SMF_GRID_LOOP(i, L.n_u) {
+    double x = 0.0;
+    const int c = (i >= L.nv) + (i >= 2 * L.nv);
+    if (c == comp) {
+      const unsigned j = (unsigned)(i - c * L.nv), n0 = (unsigned)L.N[0], n1 = (unsigned)L.N[1], r = j / n0;
+      const int g[3] = {(int)(j - r * n0), (int)(r % n1), (int)(r / n1)};
+      if (probe_colour(g, L.dim, P, cx, cy, cz) && !vel_constrained(L.N, L.faces, L.dim, g[0], g[1], g[2])) x = sqrt(DAinv[i]);
+    }
+    vc[i] = x;
+  }
+}
+__global__ void k_add_sq_cols(const double *__restrict__ y, long long ld, int cols, double *__restrict__ acc, long long n) {
+  SMF_GRID_LOOP(i, n) {
+    double s = acc[i];
+    for (int c = 0; c < cols; ++c) s += y[c * ld + i] * y[c * ld + i];
+    acc[i] = s;
+  }
+}
 __global__ void k_add_sq(const double *__restrict__ y, double *__restrict__ acc, long long n) {
   pdl_enter();
   SMF_GRID_LOOP(i, n) acc[i] += y[i] * y[i];
@@ -1072,6 +1096,25 @@ static int schur_diag_d(stokes_ctx *C, int l, double *dS) {
   const int P = 2 * d.k + 1, nz = d.dim == 3 ? P : 1;
   double *v = C->lz0, *y = C->lz1;
   SMF_CUDA_OK(cudaMemsetAsync(dS, 0, d.n_p * sizeof(double), C->s));
+  // k = 2 in 3D: many colours a launch on the Krylov space's memory (375 probes of four launches each took 20 ms of a
+  // 16^3 setup, launch-bound); deterministic contexts keep the deterministic applications below
+  if (d.dim == 3 && d.k == 2 && !C->det && !LV.rho && (d.cartesian || LV.geox)) {
+    const long long top = C->L64[C->nl - 1].d.n_u + C->L64[C->nl - 1].d.n_p, ld = (d.n_u + 31) / 32 * 32;
+    const int colours = P * P * P, cols = (int)std::min<long long>(colours, C->restart * top / ld);
+    if (cols >= 1) {
+      for (int comp = 0; comp < 3; ++comp)
+        for (int c0 = 0; c0 < colours; c0 += cols) {
+          const int nc = std::min(cols, colours - c0);
+          k_probe_vel_cols<<<dim3(vec_blocks(d.n_u), nc), kVecThreads, 0, C->s>>>(d, comp, P, c0, LV.DAinv, C->V, ld);
+          SMF_CUDA_OK(cudaMemsetAsync(C->Z, 0, (size_t)nc * ld * sizeof(double), C->s));
+          launch_cell_apply_fx(d, kApplyB, C->V, nullptr, nullptr, C->Z, LV.geox, nullptr, C->s, nc, ld);
+          k_add_sq_cols<<<vec_blocks(d.n_p), kVecThreads, 0, C->s>>>(C->Z, ld, nc, dS, d.n_p);
+          C->launches += 3;
+        }
+      SMF_CUDA_OK(cudaGetLastError());
+      return STOKES_OK;
+    }
+  }
   for (int comp = 0; comp < d.dim; ++comp)
     for (int cz = 0; cz < nz; ++cz)
       for (int cy = 0; cy < P; ++cy)
@@ -1139,49 +1182,54 @@ static int lanczos(stokes_ctx *C, int l, bool velocity, double *est) {
   int st = dot64(C, v, v, n, &nrm2);
   if (st) return st;
   k_scale<double><<<nb, kVecThreads, 0, C->s>>>(v, 1.0 / std::sqrt(nrm2), v, n);
-  SMF_CUDA_OK(cudaMemsetAsync(vprev, 0, n * sizeof(double), C->s));
-  ++C->launches;
-  std::vector<double> al, be;
-  double bprev = 0.0;
+  k_mul<double><<<nb, kVecThreads, 0, C->s>>>(sq, v, tmp, n);
+  C->launches += 2;
+  // the coefficients a_j and ||w_j||^2 stay on the device until the last step (two host round trips a step made
+  // the setup wait 480 times on three levels); the steps after an early stop below are computed and ignored
   const int steps = std::max(1, C->o.eig_iters);
+  double *da = C->lzs, *db = C->lzs + steps;
   for (int j = 0; j < steps; ++j) {
-    k_mul<double><<<nb, kVecThreads, 0, C->s>>>(sq, v, tmp, n);
-    ++C->launches;
+    if (j > 0) {
+      std::swap(vprev, v);
+      k_lz_next<<<nb, kVecThreads, 0, C->s>>>(w, db + j - 1, sq, v, tmp, n);
+      ++C->launches;
+    }
     if (velocity) {
       R.apply(l, kApplyA, tmp, nullptr, w, nullptr);
     } else {
       SMF_CUDA_OK(cudaMemsetAsync(w, 0, n * sizeof(double), C->s));
       R.S_tilde(l, tmp, w);
     }
-    k_mul<double><<<nb, kVecThreads, 0, C->s>>>(sq, w, w, n);
-    k_axpy<double><<<nb, kVecThreads, 0, C->s>>>(w, -bprev, vprev, n);
+    k_lz_w<<<kRedBlocks, kVecThreads, 0, C->s>>>(sq, w, vprev, j > 0 ? db + j - 1 : nullptr, v, n, C->partial, C->kd.ticket, da + j);
+    k_lz_a<<<kRedBlocks, kVecThreads, 0, C->s>>>(da + j, w, v, n, C->partial, C->kd.ticket, db + j);
     C->launches += 2;
-    double a;
-    st = dot64(C, w, v, n, &a);
-    if (st) return st;
-    k_axpy<double><<<nb, kVecThreads, 0, C->s>>>(w, -a, v, n);
-    ++C->launches;
-    al.push_back(a);
-    double b2;
-    st = dot64(C, w, w, n, &b2);
-    if (st) return st;
-    const double b = std::sqrt(b2);
+  }
+  std::vector<double> h(2 * steps), al, be;
+  SMF_CUDA_OK(cudaMemcpyAsync(h.data(), C->lzs, h.size() * sizeof(double), cudaMemcpyDeviceToHost, C->s));
+  SMF_CUDA_OK(cudaStreamSynchronize(C->s));
+  for (int j = 0; j < steps; ++j) {
+    const double a = h[j], b = std::sqrt(h[steps + j]);
     if (!std::isfinite(a) || !std::isfinite(b)) {
       set_error("Lanczos produced a non-finite value");
       return STOKES_EBREAKDOWN;
     }
+    al.push_back(a);
     if (j == steps - 1 || b <= 1e-14 * std::max(std::fabs(a), 1.0)) break;
     be.push_back(b);
-    std::swap(vprev, v);  // vprev <- v
-    k_scale<double><<<nb, kVecThreads, 0, C->s>>>(w, 1.0 / b, v, n);
-    ++C->launches;
-    bprev = b;
   }
   be.resize(al.size() > 0 ? al.size() - 1 : 0);
   *est = tridiag_max_eig(al, be);
   return STOKES_OK;
 }
 
+// 1 on the diagonal of the constrained velocity DoFs (K0 zero there).
+__global__ void k_identity_diag(const LevelDesc<double> L, double *__restrict__ K0, long long n0) {
+  SMF_GRID_LOOP(i, L.n_u) {
+    const long long node = i % L.nv;
+    const int gx = (int)(node % L.N[0]), gy = (int)((node / L.N[0]) % L.N[1]), gz = (int)(node / ((long long)L.N[0] * L.N[1]));
+    if (vel_constrained(L.N, L.faces, L.dim, gx, gy, gz)) K0[i * n0 + i] = 1.0;
+  }
+}
 // Dense coarse matrix K_0 by applying the FP64 operator to unit vectors, then the inverse of
 // the (bordered) matrix by Gauss-Jordan with partial pivoting, all on the device.
 static int setup_coarse(stokes_ctx *C) {
@@ -1204,18 +1252,45 @@ static int setup_coarse(stokes_ctx *C) {
   if ((st = dalloc(C, &fac, nb))) return st;
   if ((st = dalloc(C, &err, 1))) return st;
   if ((st = dalloc(C, &C->Kinv, n0 * n0))) return st;
-  for (long long j = 0; j < n0; ++j) {
-    k_unit<<<vec_blocks(n0), kVecThreads, 0, C->s>>>(e, n0, j);
-    ++C->launches;
-    R.vmult(0, e, K0 + j * n0, true);
+  if (!C->det && !R.hasC()) {
+    // every column in one launch of the point kernel (the unit vectors lie in M, which is written afterwards), and the
+    // identity rows of constrained DoFs; one at a time this took three launches a column
+    k_unit_cols64<<<dim3(vec_blocks(n0), (unsigned)n0), kVecThreads, 0, C->s>>>(M, n0, 0, n0);
+    const int mode = R.form(kApplyA | kApplyBT | kApplyB);
+    const LevelDesc<double> &d = L0.d;
+    switch (d.k) {
+      case 2: launch_cell_apply_cols_k<2, double>(d, C->tab64, mode, M, M + d.n_u, K0, K0 + d.n_u, C->s, L0.rho, (int)n0, n0); break;
+      case 3: launch_cell_apply_cols_k<3, double>(d, C->tab64, mode, M, M + d.n_u, K0, K0 + d.n_u, C->s, L0.rho, (int)n0, n0); break;
+      default: launch_cell_apply_cols_k<4, double>(d, C->tab64, mode, M, M + d.n_u, K0, K0 + d.n_u, C->s, L0.rho, (int)n0, n0); break;
+    }
+    k_identity_diag<<<vec_blocks(d.n_u), kVecThreads, 0, C->s>>>(d, K0, n0);
+    C->launches += 3;
+  } else {
+    for (long long j = 0; j < n0; ++j) {
+      k_unit<<<vec_blocks(n0), kVecThreads, 0, C->s>>>(e, n0, j);
+      ++C->launches;
+      R.vmult(0, e, K0 + j * n0, true);
+    }
   }
   k_build_augmented<<<vec_blocks((long long)nb * 2 * nb), kVecThreads, 0, C->s>>>(K0, (int)n0, L0.d.n_u, bord, M);
   ++C->launches;
-  for (int k = 0; k < nb; ++k) {
-    k_gj_pivot<<<1, 1024, 0, C->s>>>(M, nb, k, fac, err);
-    dim3 g((2 * nb + 255) / 256, nb);
-    k_gj_elim<<<g, 256, 0, C->s>>>(M, nb, k, fac);
-    C->launches += 2;
+  // small matrices: one launch a step, from one buffer into the other (above 1,024 rows every block's own scan of
+  // the pivot column would cost more than the pivot kernel)
+  if (nb <= 1024) {
+    double *O = nullptr;
+    if ((st = dalloc(C, &O, (long long)nb * 2 * nb))) return st;
+    for (int k = 0; k < nb; ++k) {
+      k_gj_step<<<std::min(nb, 304), kVecThreads, 0, C->s>>>(M, O, nb, k, err);
+      std::swap(M, O);
+      ++C->launches;
+    }
+  } else {
+    for (int k = 0; k < nb; ++k) {
+      k_gj_pivot<<<1, 1024, 0, C->s>>>(M, nb, k, fac, err);
+      dim3 g((2 * nb + 255) / 256, nb);
+      k_gj_elim<<<g, 256, 0, C->s>>>(M, nb, k, fac);
+      C->launches += 2;
+    }
   }
   k_extract_inverse<<<vec_blocks(n0 * n0), kVecThreads, 0, C->s>>>(M, nb, (int)n0, C->Kinv);
   ++C->launches;
@@ -2003,6 +2078,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
   if ((st = dalloc(C, &C->hdev, 3 * (C->restart + 2)))) return st;
   if ((st = dalloc(C, &C->partial, (long long)kRedBlocks * (C->restart + 2)))) return st;
   if ((st = dalloc(C, &C->scal, 4))) return st;
+  if ((st = dalloc(C, &C->lzs, 2 * std::max(1, C->o.eig_iters)))) return st;
   double **lz[] = {&C->lz0, &C->lz1, &C->lz2, &C->lz3, &C->sq};
   for (auto p : lz)
     if ((st = dalloc(C, p, N))) return st;

@@ -917,9 +917,10 @@ __device__ __forceinline__ void fx_group(const LevelDesc<double> &L, const doubl
 template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads, 4)
     stokes_cell_apply_fx(const LevelDesc<double> L, const double *__restrict__ u, const double *__restrict__ p,
-                         double *__restrict__ yu, double *__restrict__ yp, const int2 *__restrict__ geo, const __grid_constant__ FxCart K) {
+                         double *__restrict__ yu, double *__restrict__ yp, const int2 *__restrict__ geo, const __grid_constant__ FxCart K,
+                         const long long ld) {
   pdl_enter();
-  fx_group<MODE, CART, false>(L, u, p, yu, yp, geo, blockIdx.x, threadIdx.x >> 5, K, Fuse<double>{});
+  fx_group<MODE, CART, false>(L, column(u, ld), column(p, ld), column(yu, ld), column(yp, ld), geo, blockIdx.x, threadIdx.x >> 5, K, Fuse<double>{});
 }
 template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads, 4)
@@ -1045,8 +1046,8 @@ __global__ void k_fx_geometry(const LevelDesc<double> L, int2 *__restrict__ out)
 // Launches one mode (its own translation unit: these are long kernels).
 template <int MODE>
 int launch_fx_mode(const LevelDesc<double> &L, const double *u, const double *p, double *yu, double *yp, const void *geo,
-                   const Fuse<double> *F, cudaStream_t s) {
-  const dim3 grid((unsigned)((L.n_cells + kFxCells - 1) / kFxCells)), block(kFxThreads);
+                   const Fuse<double> *F, cudaStream_t s, int cols, long long ld) {
+  const dim3 grid((unsigned)((L.n_cells + kFxCells - 1) / kFxCells), F ? 1u : (unsigned)cols), block(kFxThreads);
   const int2 *g = static_cast<const int2 *>(geo);
   const FxCart K = L.cartesian ? fx_cart(L) : FxCart{};
   if (F) {
@@ -1056,9 +1057,9 @@ int launch_fx_mode(const LevelDesc<double> &L, const double *u, const double *p,
       launch_kernel(stokes_cell_apply_fx_fused<MODE, false>, grid, block, FxStage<MODE>::G + FxStage<MODE>::C, s, L, u, p, yu, yp, g, K, *F);
   } else {
     if (L.cartesian)
-      launch_kernel(stokes_cell_apply_fx<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K);
+      launch_kernel(stokes_cell_apply_fx<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K, ld);
     else
-      launch_kernel(stokes_cell_apply_fx<MODE, false>, grid, block, FxStage<MODE>::G + FxStage<MODE>::C, s, L, u, p, yu, yp, g, K);
+      launch_kernel(stokes_cell_apply_fx<MODE, false>, grid, block, FxStage<MODE>::G + FxStage<MODE>::C, s, L, u, p, yu, yp, g, K, ld);
   }
   return 0;
 }

@@ -3,7 +3,7 @@
 
 namespace smf {
 template int launch_fx_mode<kApplyA>(const LevelDesc<double> &, const double *, const double *, double *, double *,
-                                     const void *, const Fuse<double> *, cudaStream_t);
+                                     const void *, const Fuse<double> *, cudaStream_t, int, long long);
 template int launch_fx_mode<kApplyA | kApplyBT>(const LevelDesc<double> &, const double *, const double *, double *,
-                                                double *, const void *, const Fuse<double> *, cudaStream_t);
+                                                double *, const void *, const Fuse<double> *, cudaStream_t, int, long long);
 }  // namespace smf

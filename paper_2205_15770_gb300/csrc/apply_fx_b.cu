@@ -3,20 +3,20 @@
 
 namespace smf {
 extern template int launch_fx_mode<kApplyA>(const LevelDesc<double> &, const double *, const double *, double *,
-                                            double *, const void *, const Fuse<double> *, cudaStream_t);
+                                            double *, const void *, const Fuse<double> *, cudaStream_t, int, long long);
 extern template int launch_fx_mode<kApplyA | kApplyBT>(const LevelDesc<double> &, const double *, const double *,
                                                        double *, double *, const void *, const Fuse<double> *,
-                                                       cudaStream_t);
+                                                       cudaStream_t, int, long long);
 
 int launch_cell_apply_fx(const LevelDesc<double> &L, int mode, const double *u, const double *p, double *yu, double *yp,
-                         const void *geo, const Fuse<double> *F, cudaStream_t s) {
+                         const void *geo, const Fuse<double> *F, cudaStream_t s, int cols, long long ld) {
   if (L.dim != 3 || L.k != 2 || (!L.cartesian && !geo) || L.n_cells >= (1ll << 31)) return -1;
   switch (mode) {
-    case kApplyA: return launch_fx_mode<kApplyA>(L, u, p, yu, yp, geo, F, s);
-    case kApplyBT: return launch_fx_mode<kApplyBT>(L, u, p, yu, yp, geo, F, s);
-    case kApplyB: return launch_fx_mode<kApplyB>(L, u, p, yu, yp, geo, F, s);
-    case kApplyA | kApplyBT: return launch_fx_mode<kApplyA | kApplyBT>(L, u, p, yu, yp, geo, F, s);
-    case kApplyA | kApplyBT | kApplyB: return launch_fx_mode<kApplyA | kApplyBT | kApplyB>(L, u, p, yu, yp, geo, F, s);
+    case kApplyA: return launch_fx_mode<kApplyA>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyBT: return launch_fx_mode<kApplyBT>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyB: return launch_fx_mode<kApplyB>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyA | kApplyBT: return launch_fx_mode<kApplyA | kApplyBT>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyA | kApplyBT | kApplyB: return launch_fx_mode<kApplyA | kApplyBT | kApplyB>(L, u, p, yu, yp, geo, F, s, cols, ld);
     default: return -1;
   }
 }

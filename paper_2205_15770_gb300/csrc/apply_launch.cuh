@@ -243,6 +243,9 @@ int launch_cell_diag_k(const LevelDesc<T> &L, const Tab1D<T> *tab, T *dAs, T *dS
   template int launch_cell_apply_cols_k<KK, float>(const LevelDesc<float> &, const Tab1D<float> *, int,        \
                                                     const float *, const float *, float *, float *,           \
                                                     cudaStream_t, const float *, int, long long);               \
+  template int launch_cell_apply_cols_k<KK, double>(const LevelDesc<double> &, const Tab1D<double> *, int,     \
+                                                     const double *, const double *, double *, double *,      \
+                                                     cudaStream_t, const double *, int, long long);             \
   template int launch_cell_apply_fused_k<KK, float>(const LevelDesc<float> &, int, const float *, const float *, \
                                                      float *, float *, cudaStream_t, int, const Fuse<float> &,       \
                                                      const float *);   \

@@ -16,7 +16,7 @@ template <typename T>
 int launch_cell_apply(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
                       cudaStream_t s, int shape, const T *geo = nullptr, const T *geox = nullptr, const T *rho = nullptr,
                       const GridBarrier *det = nullptr, bool plane = false);
-// `cols` vectors at once, ld entries apart (FP32)
+// `cols` vectors at once, ld entries apart
 template <int K, typename T>
 int launch_cell_apply_cols_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
                              cudaStream_t s, const T *rho, int cols, long long ld);
@@ -56,8 +56,9 @@ inline bool cc_level_supported(int dim, int k, int cartesian, size_t elt) {
 // The fixed-point FP64 kernel (shape 5, k = 2; plain and, with F, fused launches): -1 for a level or mode
 // it does not serve.  geo: trilinear levels, the coefficients that launch_fx_geometry writes at setup
 // (fx_geometry_bytes(cells) bytes).
+// cols: plain launches on that many vectors at once, ld entries apart.
 int launch_cell_apply_fx(const LevelDesc<double> &L, int mode, const double *u, const double *p, double *yu, double *yp,
-                         const void *geo, const Fuse<double> *F, cudaStream_t s);
+                         const void *geo, const Fuse<double> *F, cudaStream_t s, int cols = 1, long long ld = 0);
 long long fx_geometry_bytes(long long cells);
 void launch_fx_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
 // The FP32 kernel with a z plane per thread (shape 5 with LevelRT::plane, k = 2): as launch_cell_apply_fx.

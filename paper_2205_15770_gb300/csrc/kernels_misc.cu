@@ -142,6 +142,49 @@ __global__ void k_gj_elim(double *__restrict__ M, int nb, int k, const double *_
     M[(long long)i * ld + j] -= f * M[(long long)k * ld + j];
 }
 
+// One Gauss-Jordan step from M into O, for small matrices: every block finds the pivot of column k itself (its nb
+// entries come from L2) and writes its rows of the swapped, scaled and eliminated matrix, one launch a step instead
+// of two and no single-block pivot kernel (nb = 403: 10 -> 4 us a step).  err: a column without a pivot.
+__global__ void k_gj_step(const double *__restrict__ M, double *__restrict__ O, int nb, int k, int *__restrict__ err) {
+  __shared__ double bv[kVecThreads];
+  __shared__ int bi[kVecThreads];
+  const int ld = 2 * nb;
+  double best = -1.0;
+  int besti = k;
+  for (int i = k + threadIdx.x; i < nb; i += blockDim.x) {
+    const double a = fabs(M[(long long)i * ld + k]);
+    if (a > best) {
+      best = a;
+      besti = i;
+    }
+  }
+  bv[threadIdx.x] = best;
+  bi[threadIdx.x] = besti;
+  __syncthreads();
+  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    if (threadIdx.x < s &&
+        (bv[threadIdx.x + s] > bv[threadIdx.x] || (bv[threadIdx.x + s] == bv[threadIdx.x] && bi[threadIdx.x + s] < bi[threadIdx.x]))) {
+      bv[threadIdx.x] = bv[threadIdx.x + s];
+      bi[threadIdx.x] = bi[threadIdx.x + s];
+    }
+    __syncthreads();
+  }
+  const int p = bi[0];
+  if (!(bv[0] > 0.0) && blockIdx.x == 0 && threadIdx.x == 0) err[0] = 1;
+  const double *piv = M + (long long)p * ld;
+  const double inv = 1.0 / piv[k];
+  for (int i = blockIdx.x; i < nb; i += gridDim.x) {
+    double *o = O + (long long)i * ld;
+    if (i == k) {
+      for (int j = threadIdx.x; j < ld; j += blockDim.x) o[j] = piv[j] * inv;
+    } else {
+      const double *r = M + (long long)(i == p ? k : i) * ld;
+      const double f = r[k];
+      for (int j = threadIdx.x; j < ld; j += blockDim.x) o[j] = r[j] - f * (piv[j] * inv);
+    }
+  }
+}
+
 // Kinv (row-major n0 x n0) = top-left block of the right half of M.
 __global__ void k_extract_inverse(const double *__restrict__ M, int nb, int n0, double *__restrict__ Kinv) {
   SMF_GRID_LOOP(idx, (long long)n0 * n0) {
@@ -298,5 +341,71 @@ __global__ void k_batch_any(const BatchCond B) {
   cudaGraphSetConditional(B.loop, any ? 1u : 0u);
 }
 
+
+}  // namespace smf
+
+namespace smf {
+
+// ---- Lanczos with its coefficients on the device ------------------------------------------------------
+// The last block to finish (ticket) adds the blocks' partial sums in a fixed order.
+__device__ __forceinline__ void finish_dot(double s, double *sh, double *partial, unsigned *ticket, double *out) {
+  __shared__ int last;
+  s = block_reduce_sum<double>(s, sh);
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = s;
+    __threadfence();
+    last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double t = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) t += __ldcg(partial + b);
+  t = block_reduce_sum<double>(t, sh);
+  if (threadIdx.x == 0) out[0] = t;
+}
+__global__ void k_lz_next(const double *__restrict__ w, const double *__restrict__ b2, const double *__restrict__ sq,
+                          double *__restrict__ v, double *__restrict__ tmp, long long n) {
+  pdl_enter();
+  const double s = 1.0 / sqrt(b2[0]);
+  SMF_GRID_LOOP(i, n) {
+    const double x = s * w[i];
+    v[i] = x;
+    tmp[i] = sq[i] * x;
+  }
+}
+__global__ void k_lz_w(const double *__restrict__ sq, double *__restrict__ w, const double *__restrict__ vprev,
+                       const double *__restrict__ b2prev, const double *__restrict__ v, long long n,
+                       double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ a) {
+  pdl_enter();
+  __shared__ double sh[32];
+  const double b = b2prev ? sqrt(b2prev[0]) : 0.0;
+  double s = 0.0;
+  SMF_GRID_LOOP(i, n) {
+    double x = sq[i] * w[i];
+    if (b2prev) x -= b * vprev[i];
+    w[i] = x;
+    s += x * v[i];
+  }
+  finish_dot(s, sh, partial, ticket, a);
+}
+__global__ void k_lz_a(const double *__restrict__ a, double *__restrict__ w, const double *__restrict__ v, long long n,
+                       double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ b2) {
+  pdl_enter();
+  __shared__ double sh[32];
+  const double al = a[0];
+  double s = 0.0;
+  SMF_GRID_LOOP(i, n) {
+    const double x = w[i] - al * v[i];
+    w[i] = x;
+    s += x * x;
+  }
+  finish_dot(s, sh, partial, ticket, b2);
+}
+
+// unit vectors j0 + blockIdx.y as columns ld entries apart
+__global__ void k_unit_cols64(double *__restrict__ e, long long n, long long j0, long long ld) {
+  SMF_GRID_LOOP(i, n) e[blockIdx.y * ld + i] = i == j0 + blockIdx.y ? 1.0 : 0.0;
+}
 
 }  // namespace smf

@@ -465,6 +465,17 @@ __global__ void k_build_augmented(const double *__restrict__ K0, int n0, long lo
                                   double *__restrict__ M);
 __global__ void k_gj_pivot(double *__restrict__ M, int nb, int k, double *__restrict__ fac, int *__restrict__ err);
 __global__ void k_gj_elim(double *__restrict__ M, int nb, int k, const double *__restrict__ fac);
+__global__ void k_gj_step(const double *__restrict__ M, double *__restrict__ O, int nb, int k, int *__restrict__ err);
+__global__ void k_unit_cols64(double *__restrict__ e, long long n, long long j0, long long ld);
+// Lanczos with its coefficients on the device: v = w / sqrt(b2), tmp = sq v;  w = sq w - sqrt(b2prev) vprev and
+// a = w . v;  w -= a v and b2 = w . w (the dot products finished by the last block, fixed order)
+__global__ void k_lz_next(const double *__restrict__ w, const double *__restrict__ b2, const double *__restrict__ sq,
+                          double *__restrict__ v, double *__restrict__ tmp, long long n);
+__global__ void k_lz_w(const double *__restrict__ sq, double *__restrict__ w, const double *__restrict__ vprev,
+                       const double *__restrict__ b2prev, const double *__restrict__ v, long long n,
+                       double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ a);
+__global__ void k_lz_a(const double *__restrict__ a, double *__restrict__ w, const double *__restrict__ v, long long n,
+                       double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ b2);
 __global__ void k_extract_inverse(const double *__restrict__ M, int nb, int n0, double *__restrict__ Kinv);
 // out = w / norm where norm = sqrt(*nrm2)
 __global__ void k_scale_by_inv_sqrt(const double *__restrict__ w, const double *__restrict__ nrm2,
