@@ -234,6 +234,12 @@ struct LevelRT {
   T *pt = nullptr, *rp = nullptr, *px = nullptr, *pd = nullptr, *ps = nullptr, *dp = nullptr;  // pressure
 };
 
+// What the setup's timing chose for a level.
+struct Tuned {
+  int shape, fshape;
+  bool plane, geo_stored, fuse;
+};
+
 struct GraphSlot {
   cudaGraphExec_t exec = nullptr;
   long long kernels = 0;
@@ -317,6 +323,7 @@ struct stokes_ctx {
   int pq_member = 0;
   bool use_graphs = true;
   bool fuse = true;  // fused smoothing where eligible (STOKES_NO_FUSE=1: the unfused path)
+  std::vector<Tuned> tuned64, tuned32;  // the setup's choices per level (empty: not timed)
   GraphSlot g32[2], g64[2];  // [x_zero]
   // FP32 cycle of level le from a zero start as an explicit matrix (setup_explicit; -1: none)
   int le = -1, ldm = 0;
@@ -1703,7 +1710,7 @@ static std::vector<double> coarsen_mean(const std::vector<double> &fm, const int
 }
 
 static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho, const double *mu_cell,
-                    const stokes_opts *opts, stokes_ctx *C) {
+                    const stokes_opts *opts, const stokes_ctx *like, stokes_ctx *C) {
   const int dim = mesh->dim, nl = mesh->n_levels;
   C->mesh = *mesh;
   if (mesh->vertices) {
@@ -2049,9 +2056,25 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
       }
     }
   }
+  // (a change of viscosities takes over the choices of the context it replaces: the same mesh, degree and forms; timing
+  // them again: gradient 16^3, which is one change and two solves, 55 -> 82 ms)
+  bool timed = false, taken = false;
   {
     const char *na = getenv("STOKES_NO_AUTOTUNE");
-    if (!(na && na[0] == '1') && !pinned && !C->det) {
+    timed = !(na && na[0] == '1') && !pinned && !C->det;
+    if (timed && like && !like->tuned64.empty()) {
+      taken = true;
+      for (int l = 0; l < nl; ++l) {
+        const Tuned &a = like->tuned64[l], &b = like->tuned32[l];
+        C->L64[l].shape = a.shape;
+        C->L64[l].fshape = a.fshape;
+        LevelRT<float> &F = C->L32[l];
+        F.shape = b.shape;
+        F.fshape = b.fshape;
+        F.plane = F.plane && b.plane;
+        if (b.geo_stored) F.geo = F.geo_stored;
+      }
+    } else if (timed) {
       for (int l = 0; l < nl; ++l) {
         if ((st = autotune_level<double>(C, C->L64[l], C->tab64))) return st;
         if ((st = autotune_level<float>(C, C->L32[l], C->tab32))) return st;
@@ -2147,18 +2170,29 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
   }
   // fused or unfused smoothing per level (STOKES_NO_AUTOTUNE=1 keeps the fused form)
   {
-    const char *na = getenv("STOKES_NO_AUTOTUNE");
     if (pinned) {
       for (int l = 0; l < nl; ++l) {
         C->L32[l].fuse = tune[2][l] != 0;
         C->L64[l].fuse = tune[3][l] != 0;
       }
-    } else if (!(na && na[0] == '1') && !C->det) {
+    } else if (taken) {
+      for (int l = 0; l < nl; ++l) {
+        C->L32[l].fuse = like->tuned32[l].fuse;
+        C->L64[l].fuse = like->tuned64[l].fuse;
+      }
+    } else if (timed) {
       for (int l = 1; l < nl; ++l) {
         if ((st = autotune_fusion<float>(C, l))) return st;
         if ((st = autotune_fusion<double>(C, l))) return st;
       }
     }
+    if (timed)
+      for (int l = 0; l < nl; ++l) {
+        const LevelRT<double> &a = C->L64[l];
+        const LevelRT<float> &b = C->L32[l];
+        C->tuned64.push_back({a.shape, a.fshape, a.plane, false, a.fuse});
+        C->tuned32.push_back({b.shape, b.fshape, b.plane, b.geo != nullptr, b.fuse});
+      }
   }
   if ((st = setup_explicit(C))) return st;
   SMF_CUDA_OK(cudaStreamSynchronize(C->s));
@@ -3229,8 +3263,9 @@ static int check_cell_orientation(const stokes_mesh *mesh) {
   return STOKES_OK;
 }
 
-int stokes_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho, const double *mu_cell,
-                 const stokes_opts *opts, void *stream, stokes_ctx **out) {
+// like: a context for the same mesh, degree and options whose timed choices are taken over, or null.
+static int setup_like(const stokes_mesh *mesh, int k, double mu, double gamma_rho, const double *mu_cell,
+                      const stokes_opts *opts, void *stream, const stokes_ctx *like, stokes_ctx **out) {
   if (!out) {
     set_error("out is NULL");
     return STOKES_EINVAL;
@@ -3273,7 +3308,7 @@ int stokes_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho, co
     cudaGetLastError();
     C->device = -1;
   }
-  int st = do_setup(mesh, k, mu, gamma_rho, mu_cell, opts, C);
+  int st = do_setup(mesh, k, mu, gamma_rho, mu_cell, opts, like, C);
   if (st == STOKES_OK) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) st = cuda_fail(e, "setup kernels", __FILE__, __LINE__);
@@ -3284,6 +3319,11 @@ int stokes_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho, co
   }
   *out = C;
   return STOKES_OK;
+}
+
+int stokes_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho, const double *mu_cell,
+                 const stokes_opts *opts, void *stream, stokes_ctx **out) {
+  return setup_like(mesh, k, mu, gamma_rho, mu_cell, opts, stream, nullptr, out);
 }
 
 int stokes_sizes(const stokes_ctx *C, int level, long long *n_u, long long *n_p) {
@@ -3598,7 +3638,7 @@ int stokes_set_viscosity(stokes_ctx *C, const double *mu_cell, void *stream) {
   // coarse inverse, captured graphs) in a fresh context, then take over its contents
   stokes_ctx *T = nullptr;
   stokes_mesh mesh = C->mesh;
-  const int st = stokes_setup(&mesh, C->k, C->mu_const, C->gamma_rho, mu_cell, &C->o, stream, &T);
+  const int st = setup_like(&mesh, C->k, C->mu_const, C->gamma_rho, mu_cell, &C->o, stream, C, &T);
   if (st != STOKES_OK) {
     C->err = g_last_error;
     return st;

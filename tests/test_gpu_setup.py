@@ -64,3 +64,22 @@ def test_lanczos_beyond_the_dimension(dim, n):
     lam = torch.linalg.eigvalsh((s[:, None] * A * s).cpu()).max().item()
     # an extreme Ritz value, its error the square of the residual's: far below the tolerance after all the dimensions
     assert abs(S.level_params(1)["beta_A"] - lam) <= 1e-8 * lam
+
+
+@pytest.mark.parametrize("fp32", [True, False])
+def test_change_of_viscosities_keeps_the_tuned_choices(fp32):
+    from paper_2205_15770_gb300 import StokesMG
+    n, rng = (8, 8, 8), np.random.default_rng(5)
+    mu = [np.exp(rng.standard_normal(512)) for _ in range(3)]
+    kw = dict(vertices=W.perturbed_vertices(3, n, seed=1), kA=1, kS=1, vcycle_fp32=fp32)
+    S = StokesMG(3, n, 3, mu_cell=mu[0], **kw)
+    tuned = [(S.launch_shapes(p), S.fused_levels(p), S.geometry_stored(p)) for p in (32, 64)]
+    S.set_launch_shape(2, 1, 64)  # a caller's shape lasts until the next change of viscosities
+    for m in mu[1:]:
+        S.set_viscosity(m)
+        assert [(S.launch_shapes(p), S.fused_levels(p), S.geometry_stored(p)) for p in (32, 64)] == tuned
+        F = StokesMG(3, n, 3, mu_cell=m, **kw)
+        x = torch.as_tensor(rng.uniform(-1, 1, S.size()), device="cuda")
+        ref = F.vcycle(x)
+        # FP64 evaluations of one map by kernels that may differ: a few hundred roundings
+        assert (S.vcycle(x) - ref).norm().item() <= 1e-13 * ref.norm().item()
