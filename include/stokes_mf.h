@@ -35,6 +35,8 @@
  *  - STOKES_HOST_KRYLOV=1: the FGMRES iterations driven from the host (stokes_krylov_mode).
  *  - STOKES_BATCH_QUEUE=1: the batch's FP32 cycles in the persistent work-queue kernel.
  *  - STOKES_NO_EXPLICIT=1: the FP32 cycle of the small coarse levels by launches, not as an explicit matrix.
+ *  - STOKES_NO_SCHUR_MATRIX=1: S~ = B A^-1_hat B^T by its applications on every level, not as an explicit matrix
+ *    (k = 2, kA = 1).
  *  - STOKES_NO_PLANE=1: FP32 launch shape 5 is the cell-component kernel, never the plane kernel (k = 2).
  *  - STOKES_GEO=none: no stored per-point geometry (stokes_get_geometry_stored).
  *    STOKES_C_MATRIX=none: the stabilisation block C on the fly instead of stored element matrices.

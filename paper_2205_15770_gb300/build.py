@@ -20,7 +20,7 @@ LIB = os.path.join(HERE, "libstokes_mf.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 SOURCES = ["api.cu", "kernels_misc.cu", "apply_k2.cu", "apply_k3.cu", "apply_k4.cu", "apply_cc_k2.cu", "apply_cc_k3.cu",
-           "apply_fx_a.cu", "apply_fx_b.cu", "apply_pl.cu",
+           "apply_fx_a.cu", "apply_fx_b.cu", "apply_pl.cu", "schur.cu",
            "host_tables.cpp"]
 
 

@@ -15,6 +15,7 @@
 #include "host_tables.h"
 #include "queue.h"
 #include "transfer.cuh"
+#include "schur.cuh"
 #include "vec.cuh"
 
 namespace smf {
@@ -227,6 +228,7 @@ struct LevelRT {
   bool plane = false;      // FP32 shape 5: the plane kernel (false: the cell-component kernel)
   const T *rho = nullptr;  // per-cell density of the gamma rho mass term (null: rho = 1)
   const T *Ce = nullptr;   // packed element matrices of the stabilisation block C (null: on the fly)
+  const T *sm = nullptr;   // explicit S~ (schur.cuh; null: B, A^-1_hat and B^T applied one after the other)
   T *DAinv = nullptr, *DSinv = nullptr;
   T *x = nullptr, *b = nullptr, *r = nullptr, *kx = nullptr;                   // full vectors
   T *tu = nullptr, *ru = nullptr, *uhat = nullptr, *cx = nullptr, *cd = nullptr, *ct = nullptr;  // velocity
@@ -422,7 +424,7 @@ struct Runner {
   cudaStream_t s;
   std::vector<LevelRT<T>> &L;
   const Tab1D<T> *tab;
-  int cols = 1;      // vectors handled by every launch, ld entries apart (setup_explicit; FP32, unfused forms)
+  int cols = 1;      // vectors handled by every launch, ld entries apart (setup; unfused forms)
   long long ld = 0;
   explicit Runner(stokes_ctx *c) : C(c), s(c->s), L(levels<T>(c)), tab(tables<T>(c)) {}
   // several columns on their own work vectors
@@ -495,16 +497,24 @@ struct Runner {
       o.items = pq_items(o);
       return;
     }
-    if constexpr (std::is_same<T, float>::value) {
-      if (cols > 1) {
-        switch (L[l].d.k) {
-          case 2: launch_cell_apply_cols_k<2, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
-          case 3: launch_cell_apply_cols_k<3, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
-          default: launch_cell_apply_cols_k<4, T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].rho, cols, ld); break;
-        }
-        note();
-        return;
+    if (cols > 1) {
+      const int m = form(mode);
+      bool done = false;
+      if (!L[l].rho) {
+        if constexpr (sizeof(T) == 8)
+          done = launch_cell_apply_fx(L[l].d, m, u, p, yu, yp, L[l].geox, nullptr, s, cols, ld) == 0;
+        else
+          done = L[l].plane && launch_cell_apply_pl(L[l].d, m, u, p, yu, yp, L[l].geox, nullptr, s, cols, ld) == 0;
       }
+      if (!done) {
+        switch (L[l].d.k) {
+          case 2: launch_cell_apply_cols_k<2, T>(L[l].d, tab, m, u, p, yu, yp, s, L[l].rho, cols, ld); break;
+          case 3: launch_cell_apply_cols_k<3, T>(L[l].d, tab, m, u, p, yu, yp, s, L[l].rho, cols, ld); break;
+          default: launch_cell_apply_cols_k<4, T>(L[l].d, tab, m, u, p, yu, yp, s, L[l].rho, cols, ld); break;
+        }
+      }
+      note();
+      return;
     }
     launch_cell_apply<T>(L[l].d, tab, form(mode), u, p, yu, yp, s, L[l].shape, L[l].geo, L[l].geox, L[l].rho,
                          C->det ? &C->gb : nullptr, L[l].plane);
@@ -563,6 +573,24 @@ struct Runner {
     cheb_init_op(l, n, a, b, sr, Dinv, (T)cc.c0, rb, (T *)nullptr, xb, (const T *)nullptr, T(0), (T *)nullptr, (T *)nullptr, za,
                  zb);
     for (int j = 1; j <= kd; ++j) {
+      if (!velocity && j == kd && R.sm && !rec() && !base) {  // the last step in S~'s epilogue
+        StencilIn<T> in;
+        in.v[0] = xb;
+        in.c[0] = T(1);
+        in.n = 1;
+        StencilOut<T> o;
+        o.r = rb;
+        o.d = j == 1 ? nullptr : db;
+        o.x = xb;
+        o.Dinv = Dinv;
+        o.c1 = (T)cc.c1[j];
+        o.c2 = (T)cc.c2[j];
+        o.scale = scale;
+        o.out = out;
+        o.acc = acc;
+        stencil(l, in, o);
+        return;
+      }
       if (velocity)
         apply_nz(l, kApplyA, xb, nullptr, tb, nullptr);
       else
@@ -615,9 +643,23 @@ struct Runner {
     vecp(k_cheb_step<T, 1>, k_cheb_step<T, VW>, {r, t, Dinv, d, x, base, final_out, acc_out}, n, r, t, Dinv, c1, c2,
          d, x, base, fscale, final_out, acc_out, flags, n, ld);
   }
+  void stencil(int l, const StencilIn<T> &in, const StencilOut<T> &o) {
+    launch_stencil<T>(L[l].d, L[l].sm, in, o, cols, ld, s);
+    note();
+  }
   // y = B A^-1_hat B^T q   (y zero on entry)
   void S_tilde(int l, const T *q, T *y) {
     LevelRT<T> &R = L[l];
+    if (R.sm && !rec()) {
+      StencilIn<T> in;
+      in.v[0] = q;
+      in.c[0] = T(1);
+      in.n = 1;
+      StencilOut<T> o;
+      o.t = y;
+      stencil(l, in, o);
+      return;
+    }
     apply_nz(l, kApplyBT, nullptr, q, R.tu, nullptr);
     cheb(l, true, true, R.tu, nullptr, R.tu, nullptr, T(1), nullptr, T(1), R.au, nullptr);
     apply_nz(l, kApplyB, R.au, nullptr, nullptr, y);
@@ -852,6 +894,23 @@ struct Runner {
     // dp = tau Cheb(S~, D_S, k_S)(pt - g); each S~ x_j = B A^-1_hat B^T x_j
     for (int j = 1; j <= kS + 1; ++j) {
       const bool last = j == kS + 1;
+      if (!last && R.sm) {  // t_j from the explicit S~: one launch for three
+        StencilIn<T> in;
+        in.d = R.DSinv;
+        in.v[0] = R.pt;
+        in.c[0] = (T)X[j][0];
+        in.v[1] = g;
+        in.c[1] = (T)-X[j][0];
+        for (int i = 1; i < j; ++i) {
+          in.v[1 + i] = psb(l, i - 1);
+          in.c[1 + i] = (T)X[j][i];
+        }
+        in.n = j + 1;
+        StencilOut<T> o;
+        o.t = psb(l, j - 1);
+        stencil(l, in, o);
+        continue;
+      }
       const int prev = pr;
       pr = 1 - pr;
       const double sc = last ? tau : 1.0;
@@ -1588,6 +1647,80 @@ static int autotune_fusion(stokes_ctx *C, int l) {
   return zero_level_work(C, L);
 }
 
+// S~ of the levels above the coarsest as its stencil matrix (k = 2, k_A = 1, C = 0).  A
+// smoothing step applies S~ k_S times through B^T, A, B and the vector updates between them (fused: three
+// launches, unfused: six); the matrix takes one launch that reads 343 (2D: 49) entries a row: cycle 32^3 FP32
+// 926 -> 777 us, 24x16x8 FP64 808 -> 620, 128^2 FP32 421 -> 327, two steps 20x24x12 FP64 280 -> 207.
+// Built by probing: one column per colour of nodes that no row sees twice (7^dim), several columns a launch.  Its
+// entries carry the rounding of the applications they come from.  The lines: in the cycle's precision kSchurBytes a
+// level (64^3 FP32, 377 MB: cycle 2.97 -> 2.60 ms); the other precision (FP64 smoothing with an FP32 cycle or the
+// reverse) up to kSchurOther, where 343 probes take about 10 ms.  A 32^3 setup takes 0.24 s with the matrices and
+// 0.19 without.  STOKES_NO_SCHUR_MATRIX=1 keeps the applications.
+template <typename T>
+constexpr long long kSchurBytes = sizeof(T) == 4 ? 512ll << 20 : 128ll << 20;
+constexpr long long kSchurOther = 32ll << 20;
+constexpr long long kSchurWork = 256ll << 20;  // work vectors of the columns
+template <typename T>
+static int setup_schur(stokes_ctx *C) {
+  const char *off = getenv("STOKES_NO_SCHUR_MATRIX");
+  if ((off && off[0] == '1') || C->k != 2 || C->o.kA != 1 || C->o.kS < 1 || C->det || C->c_mass != 0.0 || C->c_grad != 0.0)
+    return STOKES_OK;
+  std::vector<LevelRT<T>> &LV = levels<T>(C);
+  const long long limit = (sizeof(T) == 4) == (C->o.vcycle_fp32 != 0) ? kSchurBytes<T> : kSchurOther;
+  constexpr int NB = 7;
+  const auto ldv = [&](int l) { return (LV[l].d.n_u + 63) / 64 * 64; };
+  long long need = 0;
+  int top = 0;
+  for (int l = 1; l < C->nl; ++l) {
+    if (stencil_rows(LV[l].d.n_p) * stencil_entries(C->dim) * (long long)sizeof(T) > limit) break;
+    const long long col = NB * ldv(l) * (long long)sizeof(T);
+    need = std::max(need, std::max(col, std::min(kSchurWork / col, (long long)stencil_colours(LV[l].d)) * col));
+    top = l;
+  }
+  T *mem = nullptr;
+  if (top < 1) return STOKES_OK;
+  if (cudaMalloc((void **)&mem, (size_t)need) != cudaSuccess) {
+    cudaGetLastError();
+    return STOKES_OK;  // no room: the applications stay
+  }
+  for (int l = 1; l <= top; ++l) {
+    const LevelDesc<T> &d = LV[l].d;
+    T *M = nullptr;
+    size_t free_b = 0, total_b = 0;
+    SMF_CUDA_OK(cudaMemGetInfo(&free_b, &total_b));
+    const long long entries = stencil_rows(d.n_p) * stencil_entries(C->dim);
+    if (entries * (long long)sizeof(T) > (long long)(free_b / 4) || dalloc(C, &M, entries) != STOKES_OK) break;
+    std::vector<LevelRT<T>> Lb(LV.begin(), LV.begin() + l + 1);
+    const long long ld = ldv(l);
+    const int colours = stencil_colours(d);
+    const int cols = (int)std::min<long long>(colours, need / (NB * ld * (long long)sizeof(T)));
+    cudaMemsetAsync(mem, 0, (size_t)NB * cols * ld * sizeof(T), C->s);
+    T *v[NB];
+    for (int i = 0; i < NB; ++i) v[i] = mem + i * cols * ld;
+    LevelRT<T> &R = Lb[l];
+    R.tu = v[0];
+    R.r2 = v[1];
+    R.cx2 = v[2];
+    R.ct2 = v[3];
+    R.au = v[4];
+    for (int c0 = 0; c0 < colours; c0 += cols) {
+      const int nc = std::min(cols, colours - c0);
+      Runner<T> run(C, Lb, nc, ld);
+      launch_stencil_probe(d, c0, nc, ld, v[5], C->s);
+      if (c0 > 0) cudaMemsetAsync(v[6], 0, (size_t)nc * ld * sizeof(T), C->s);
+      run.S_tilde(l, v[5], v[6]);
+      launch_stencil_store(d, c0, nc, ld, (const T *)v[6], M, C->s);
+      C->launches += 2;
+    }
+    LV[l].sm = M;
+  }
+  const cudaError_t e = cudaStreamSynchronize(C->s);  // (also: the matrix is read ahead of a launch's dependencies)
+  cudaFree(mem);
+  SMF_CUDA_OK(e);
+  SMF_CUDA_OK(cudaGetLastError());
+  return STOKES_OK;
+}
+
 // The FP32 cycle of a small level below the finest as an explicit matrix.  From a zero start the gamma
 // recursive calls are linear in the right-hand side, x_l = M b_l, and on a small level their ~40 (2D: per
 // level) dependent launches of 2-4 us cost far more than reading M: 4^3 and the 2^3 coarse solve 130-156 us
@@ -2167,6 +2300,10 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
   for (int l = 0; l < nl; ++l) {
     if ((st = zero_level_work(C, C->L64[l]))) return st;
     if ((st = zero_level_work(C, C->L32[l]))) return st;
+  }
+  if (!like) {  // (for a change of viscosities the matrices would cost what its few solves gain)
+    if ((st = setup_schur<float>(C))) return st;
+    if ((st = setup_schur<double>(C))) return st;
   }
   // fused or unfused smoothing per level (STOKES_NO_AUTOTUNE=1 keeps the fused form)
   {

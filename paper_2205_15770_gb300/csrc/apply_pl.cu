@@ -4,14 +4,14 @@
 namespace smf {
 
 int launch_cell_apply_pl(const LevelDesc<float> &L, int mode, const float *u, const float *p, float *yu, float *yp,
-                         const void *geo, const Fuse<float> *F, cudaStream_t s) {
+                         const void *geo, const Fuse<float> *F, cudaStream_t s, int cols, long long ld) {
   if (L.dim != 3 || L.k != 2 || (!L.cartesian && !geo) || L.n_cells >= (1ll << 31)) return -1;
   switch (mode) {
-    case kApplyA: return launch_pl_mode<kApplyA>(L, u, p, yu, yp, geo, F, s);
-    case kApplyBT: return launch_pl_mode<kApplyBT>(L, u, p, yu, yp, geo, F, s);
-    case kApplyB: return launch_pl_mode<kApplyB>(L, u, p, yu, yp, geo, F, s);
-    case kApplyA | kApplyBT: return launch_pl_mode<kApplyA | kApplyBT>(L, u, p, yu, yp, geo, F, s);
-    case kApplyA | kApplyBT | kApplyB: return launch_pl_mode<kApplyA | kApplyBT | kApplyB>(L, u, p, yu, yp, geo, F, s);
+    case kApplyA: return launch_pl_mode<kApplyA>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyBT: return launch_pl_mode<kApplyBT>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyB: return launch_pl_mode<kApplyB>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyA | kApplyBT: return launch_pl_mode<kApplyA | kApplyBT>(L, u, p, yu, yp, geo, F, s, cols, ld);
+    case kApplyA | kApplyBT | kApplyB: return launch_pl_mode<kApplyA | kApplyBT | kApplyB>(L, u, p, yu, yp, geo, F, s, cols, ld);
     default: return -1;
   }
 }

@@ -79,9 +79,10 @@ __device__ __forceinline__ void pl_group(const LevelDesc<float> &L, const float 
 template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads)
     stokes_cell_apply_pl(const LevelDesc<float> L, const float *__restrict__ u, const float *__restrict__ p,
-                         float *__restrict__ yu, float *__restrict__ yp, const float4 *__restrict__ geo, const __grid_constant__ PlCart K) {
+                         float *__restrict__ yu, float *__restrict__ yp, const float4 *__restrict__ geo, const __grid_constant__ PlCart K,
+                         const long long ld) {
   pdl_enter();
-  pl_group<MODE, CART, false>(L, u, p, yu, yp, geo, blockIdx.x, threadIdx.x >> 5, K, Fuse<float>{});
+  pl_group<MODE, CART, false>(L, column(u, ld), column(p, ld), column(yu, ld), column(yp, ld), geo, blockIdx.x, threadIdx.x >> 5, K, Fuse<float>{});
 }
 template <int MODE, bool CART>
 __global__ void __launch_bounds__(kFxThreads)
@@ -145,8 +146,8 @@ __global__ void k_pl_geometry(const LevelDesc<double> L, float4 *__restrict__ ou
 
 template <int MODE>
 static int launch_pl_mode(const LevelDesc<float> &L, const float *u, const float *p, float *yu, float *yp, const void *geo,
-                          const Fuse<float> *F, cudaStream_t s) {
-  const dim3 grid((unsigned)((L.n_cells + kFxCells - 1) / kFxCells)), block(kFxThreads);
+                          const Fuse<float> *F, cudaStream_t s, int cols, long long ld) {
+  const dim3 grid((unsigned)((L.n_cells + kFxCells - 1) / kFxCells), F ? 1u : (unsigned)cols), block(kFxThreads);
   const float4 *g = static_cast<const float4 *>(geo);
   const PlCart K = L.cartesian ? pl_cart(L) : PlCart{};
   if (F) {
@@ -156,9 +157,10 @@ static int launch_pl_mode(const LevelDesc<float> &L, const float *u, const float
       launch_kernel(stokes_cell_apply_pl_fused<MODE, false>, grid, block, PlStage<MODE>::G + PlStage<MODE>::C, s, L, u, p, yu, yp, g, K, *F);
   } else {
     if (L.cartesian)
-      launch_kernel(stokes_cell_apply_pl<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K);
+      launch_kernel(stokes_cell_apply_pl<MODE, true>, grid, block, 0, s, L, u, p, yu, yp, g, K, ld);
     else
-      launch_kernel(stokes_cell_apply_pl<MODE, false>, grid, block, PlStage<MODE>::G + PlStage<MODE>::C, s, L, u, p, yu, yp, g, K);
+      launch_kernel(stokes_cell_apply_pl<MODE, false>, grid, block, PlStage<MODE>::G + PlStage<MODE>::C, s, L, u, p, yu, yp, g, K,
+                    ld);
   }
   return 0;
 }

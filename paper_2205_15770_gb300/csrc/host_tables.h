@@ -63,7 +63,7 @@ long long fx_geometry_bytes(long long cells);
 void launch_fx_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
 // The FP32 kernel with a z plane per thread (shape 5 with LevelRT::plane, k = 2): as launch_cell_apply_fx.
 int launch_cell_apply_pl(const LevelDesc<float> &L, int mode, const float *u, const float *p, float *yu, float *yp,
-                         const void *geo, const Fuse<float> *F, cudaStream_t s);
+                         const void *geo, const Fuse<float> *F, cudaStream_t s, int cols = 1, long long ld = 0);
 long long pl_geometry_bytes(long long cells);
 void launch_pl_geometry(const LevelDesc<double> &L, void *out, cudaStream_t s);
 template <int K, typename T>

@@ -143,8 +143,8 @@ __global__ void k_gj_elim(double *__restrict__ M, int nb, int k, const double *_
 }
 
 // One Gauss-Jordan step from M into O, for small matrices: every block finds the pivot of column k itself (its nb
-// entries come from L2) and writes its rows of the swapped, scaled and eliminated matrix, one launch a step instead
-// of two and no single-block pivot kernel (nb = 403: 10 -> 4 us a step).  err: a column without a pivot.
+// entries come from L2) and writes its rows of the swapped, scaled and eliminated matrix: one launch a step (7.4 us with
+// 403 rows) instead of a single-block pivot kernel and an elimination.  err: a column without a pivot.
 __global__ void k_gj_step(const double *__restrict__ M, double *__restrict__ O, int nb, int k, int *__restrict__ err) {
   __shared__ double bv[kVecThreads];
   __shared__ int bi[kVecThreads];
