@@ -2435,16 +2435,17 @@ static void krylov_post(stokes_ctx *C, cudaGraphConditionalHandle cond, bool set
   R64.apply_nz(top, kApplyA | kApplyBT | kApplyB, C->zcur, C->zcur + Lt.n_u, C->w, C->w + Lt.n_u);
   R64.applyC(top, C->zcur + Lt.n_u, C->w + Lt.n_u, -1.0);
   // CGS2 (two passes) and ||w||^2, each dot set with its final sums in the same launch
-  for (int pass = 0; pass < 2; ++pass) {
-    k_mdot_final_cnt<<<kRedBlocks, kVecThreads, 0, C->s>>>(C->V, N, ctl, 1, C->w, N, C->partial, C->kd.ticket,
-                                                           C->hdev + pass * (m + 2));
-    k_maxpy_cnt<<<nb, kVecThreads, 0, C->s>>>(C->V, N, ctl, 1, C->hdev + pass * (m + 2), C->w, N, -1.0);
-  }
-  k_mdot_final_cnt<<<kRedBlocks, kVecThreads, 0, C->s>>>(nullptr, N, nullptr, 0, C->w, N, C->partial, C->kd.ticket,
-                                                         C->hdev + 2 * (m + 2));
+  const auto dots = [&](double *h) {
+    k_mdot_final_cnt<<<kRedBlocks, kVecThreads, 0, C->s>>>(C->V, N, ctl, 1, C->w, N, C->partial, C->kd.ticket, h);
+  };
+  dots(C->hdev);
+  k_maxpy_cnt<<<nb, kVecThreads, 0, C->s>>>(C->V, N, ctl, 1, C->hdev, C->w, N, -1.0);
+  dots(C->hdev + m + 2);
+  k_maxpy_norm_cnt<<<2 * kRedBlocks, kVecThreads, 0, C->s>>>(C->V, N, ctl, 1, C->hdev + m + 2, C->w, N, C->partial,
+                                                             C->kd.ticket, C->hdev + 2 * (m + 2));
   k_scale_to_slot<<<nb, kVecThreads, 0, C->s>>>(C->w, C->hdev + 2 * (m + 2), C->V, N, ctl, N);
   k_fgmres_givens<<<1, 32, 0, C->s>>>(C->kd, cond, set_cond ? 1 : 0);
-  C->cap_count += 8;
+  C->cap_count += 7;
 }
 
 // Builds the device Krylov graph: a conditional while node whose body is krylov_body.  Returns

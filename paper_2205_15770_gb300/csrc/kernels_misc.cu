@@ -47,6 +47,7 @@ __global__ void k_maxpy(const double *__restrict__ V, long long ldv, int nvec, c
   pdl_enter();
   SMF_GRID_LOOP(i, n) {
     double s = 0.0;
+#pragma unroll 4
     for (int j = 0; j < nvec; ++j) s += h[j] * V[(long long)j * ldv + i];
     w[i] += sign * s;
   }
@@ -211,33 +212,67 @@ __global__ void k_mdot_partial_cnt(const double *__restrict__ V, long long ldv, 
   }
 }
 
+// The sums over a warp of eight values a lane, value (lane >> 2) in the result: each exchange also halves the values a
+// lane still holds, 9 additions instead of the 40 of eight separate reductions (a warp's FP64 addition occupies an
+// SM's FP64 unit for 19 clocks).
+__device__ __forceinline__ double warp_sum8(double a[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int w = 4, m = 16; w >= 1; w >>= 1, m >>= 1) {
+    const bool hi = lane & m;
+#pragma unroll
+    for (int k = 0; k < w; ++k) {
+      const double send = hi ? a[k] : a[k + w], keep = hi ? a[k + w] : a[k];
+      a[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+  }
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+  a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+  return a[0];
+}
+// h[j] = V_j . w, j < ctl[0] + add, finished by the last block in a fixed order.  Bound by the FP64 unit (a
+// multiply-add an entry, 1.8 us a vector of 859,000) and by reading V: eight vectors a pass over w, so that their
+// loads are independent, their sums share the reduction, and w is read once for all of them.  (A vector at a time took
+// 6.9 us for one and 33 for six.)
 __global__ void k_mdot_final_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
                                  const double *__restrict__ w, long long n, double *__restrict__ partial,
                                  unsigned *__restrict__ ticket, double *__restrict__ out) {
   pdl_enter();
-  __shared__ double sh[32];
+  constexpr int NW = kVecThreads / 32;
+  __shared__ double sh[NW][8];
   __shared__ int last;
-  const int nvec = ctl ? ctl[0] + add : 1;
-  for (int j = 0; j < nvec; ++j) {
-    const double *v = ctl ? V + (long long)j * ldv : w;
-    double s = 0.0;
-    SMF_GRID_LOOP(i, n) s += v[i] * w[i];
-    s = block_reduce_sum<double>(s, sh);
-    if (threadIdx.x == 0) partial[(long long)j * gridDim.x + blockIdx.x] = s;
+  const int nvec = ctl[0] + add, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int j0 = 0; j0 < nvec; j0 += 8) {
+    double s[8] = {};
+    const double *v = V + (long long)j0 * ldv;
+    SMF_GRID_LOOP(i, n) {
+      const double wi = w[i];
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (j0 + c < nvec) s[c] += v[c * ldv + i] * wi;
+    }
+    const double t = warp_sum8(s);
+    if ((lane & 3) == 0) sh[warp][lane >> 2] = t;
+    __syncthreads();
+    if (threadIdx.x < 8 && j0 + (int)threadIdx.x < nvec) {
+      double b = 0.0;
+#pragma unroll
+      for (int k = 0; k < NW; ++k) b += sh[k][threadIdx.x];
+      partial[(long long)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = b;
+      __threadfence();  // this block's partial sums before its ticket
+    }
+    __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    __threadfence();  // this block's partial sums before its ticket
-    last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;  // the counter wraps back to 0
-  }
+  if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;  // the counter wraps back to 0
   __syncthreads();
   if (!last) return;
   __threadfence();
   const int nparts = gridDim.x;
-  for (int j = 0; j < nvec; ++j) {
+  for (int j = warp; j < nvec; j += NW) {
     double s = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += __ldcg(partial + (long long)j * nparts + b);
-    s = block_reduce_sum<double>(s, sh);
-    if (threadIdx.x == 0) out[j] = s;
+    for (int b = lane; b < nparts; b += 32) s += __ldcg(partial + (long long)j * nparts + b);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) out[j] = s;
   }
 }
 
@@ -259,15 +294,24 @@ __global__ void k_maxpy_cnt(const double *__restrict__ V, long long ldv, const i
   const int nvec = ctl[0] + add;
   SMF_GRID_LOOP(i, n) {
     double s = 0.0;
+#pragma unroll 4
     for (int j = 0; j < nvec; ++j) s += h[j] * V[(long long)j * ldv + i];
     w[i] += sign * s;
   }
 }
 
+// 1 / sqrt(x), by one thread of the block: by all of them the division and the root were the kernel (859,000 entries:
+// 24 us on the FP64 unit, for 14 MB).
+__device__ __forceinline__ double block_rsqrt(double x) {
+  __shared__ double s;
+  if (threadIdx.x == 0) s = 1.0 / sqrt(x);
+  __syncthreads();
+  return s;
+}
 __global__ void k_scale_to_slot(const double *__restrict__ w, const double *__restrict__ nrm2, double *__restrict__ V,
                                 long long ldv, const int *__restrict__ ctl, long long n) {
   pdl_enter();
-  const double s = 1.0 / sqrt(nrm2[0]);
+  const double s = block_rsqrt(nrm2[0]);
   double *out = V + (long long)(ctl[0] + 1) * ldv;
   SMF_GRID_LOOP(i, n) out[i] = s * w[i];
 }
@@ -364,10 +408,28 @@ __device__ __forceinline__ void finish_dot(double s, double *sh, double *partial
   t = block_reduce_sum<double>(t, sh);
   if (threadIdx.x == 0) out[0] = t;
 }
+// w -= sum_j h_j V_j over j < ctl[0] + add, and nrm2 = w . w in the same pass (finished by the last block).
+__global__ void k_maxpy_norm_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
+                                 const double *__restrict__ h, double *__restrict__ w, long long n,
+                                 double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ nrm2) {
+  pdl_enter();
+  __shared__ double sh[32];
+  const int nvec = ctl[0] + add;
+  double q = 0.0;
+  SMF_GRID_LOOP(i, n) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int j = 0; j < nvec; ++j) s += h[j] * V[(long long)j * ldv + i];
+    const double x = w[i] - s;
+    w[i] = x;
+    q += x * x;
+  }
+  finish_dot(q, sh, partial, ticket, nrm2);
+}
 __global__ void k_lz_next(const double *__restrict__ w, const double *__restrict__ b2, const double *__restrict__ sq,
                           double *__restrict__ v, double *__restrict__ tmp, long long n) {
   pdl_enter();
-  const double s = 1.0 / sqrt(b2[0]);
+  const double s = block_rsqrt(b2[0]);
   SMF_GRID_LOOP(i, n) {
     const double x = s * w[i];
     v[i] = x;
@@ -379,7 +441,10 @@ __global__ void k_lz_w(const double *__restrict__ sq, double *__restrict__ w, co
                        double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ a) {
   pdl_enter();
   __shared__ double sh[32];
-  const double b = b2prev ? sqrt(b2prev[0]) : 0.0;
+  __shared__ double bs;
+  if (threadIdx.x == 0) bs = b2prev ? sqrt(b2prev[0]) : 0.0;
+  __syncthreads();
+  const double b = bs;
   double s = 0.0;
   SMF_GRID_LOOP(i, n) {
     double x = sq[i] * w[i];

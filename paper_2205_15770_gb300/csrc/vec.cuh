@@ -466,6 +466,9 @@ __global__ void k_build_augmented(const double *__restrict__ K0, int n0, long lo
 __global__ void k_gj_pivot(double *__restrict__ M, int nb, int k, double *__restrict__ fac, int *__restrict__ err);
 __global__ void k_gj_elim(double *__restrict__ M, int nb, int k, const double *__restrict__ fac);
 __global__ void k_gj_step(const double *__restrict__ M, double *__restrict__ O, int nb, int k, int *__restrict__ err);
+__global__ void k_maxpy_norm_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
+                                 const double *__restrict__ h, double *__restrict__ w, long long n,
+                                 double *__restrict__ partial, unsigned *__restrict__ ticket, double *__restrict__ nrm2);
 __global__ void k_unit_cols64(double *__restrict__ e, long long n, long long j0, long long ld);
 // Lanczos with its coefficients on the device: v = w / sqrt(b2), tmp = sq v;  w = sq w - sqrt(b2prev) vprev and
 // a = w . v;  w -= a v and b2 = w . w (the dot products finished by the last block, fixed order)
