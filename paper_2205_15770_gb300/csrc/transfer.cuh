@@ -124,10 +124,14 @@ __global__ void k_restrict(const LevelDesc<T> F, const LevelDesc<T> C, const Xfe
   }
 }
 
-// Prolongation row of fine DoF i: (P in)_i.
+// Prolongation row of fine DoF i: (P in)_i.  Bound by load latency: the rows of the three tables (at most k + 1
+// entries each) are read into registers first, so that the loops over them have constant bounds and the loads of
+// the terms are independent.  (Loops over the tables' counts, each term behind its own index load, took 28.1 us
+// for 859,000 DoFs in FP32, against 17.2.)
 template <typename T, int W, bool COH = false>
 __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDesc<T> &C, const XferTabs<T> &X,
                                            const T *in, long long i) {
+  constexpr int PW = (W - 1) / 4 + 1;
   const bool vel = i < F.n_u;
   const int sp = vel ? 0 : 1;
   const int *Nc = vel ? C.N : C.Pn, *Nf = vel ? F.N : F.Pn;
@@ -136,15 +140,32 @@ __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDes
   const T *src = in + (vel ? comp * C.nv : C.n_u);
   const Xfer1D<T> &ax = X.p[sp][0], &ay = X.p[sp][1], &az = X.p[sp][2];
   const int n0 = ax.cnt[g0], n1 = ay.cnt[g1], n2 = az.cnt[g2];
+  if (n0 == 0) return T(0);
+  int i0[PW], i1[PW];
+  T w0[PW], w1[PW];
+#pragma unroll
+  for (int a = 0; a < PW; ++a) {
+    i0[a] = ax.idx[g0 * W + (a < n0 ? a : 0)];  // past the row: its first node again, with weight 0
+    w0[a] = a < n0 ? ax.w[g0 * W + a] : T(0);
+    i1[a] = a < n1 ? ay.idx[g1 * W + a] : 0;
+    w1[a] = a < n1 ? ay.w[g1 * W + a] : T(0);
+  }
   T s = T(0);
-  for (int a2 = 0; a2 < n2; ++a2) {
-    const int G2 = az.idx[g2 * W + a2];
-    const T w2 = az.w[g2 * W + a2];
-    for (int a1 = 0; a1 < n1; ++a1) {
-      const T *row = src + ((long long)G2 * Nc[1] + ay.idx[g1 * W + a1]) * Nc[0];
-      T r = T(0);
-      for (int a0 = 0; a0 < n0; ++a0) r += ax.w[g0 * W + a0] * ld_in<COH>(row + ax.idx[g0 * W + a0]);
-      s += w2 * ay.w[g1 * W + a1] * r;
+#pragma unroll
+  for (int a2 = 0; a2 < PW; ++a2) {
+    if (a2 < n2) {
+      const int G2 = az.idx[g2 * W + a2];
+      const T w2 = az.w[g2 * W + a2];
+#pragma unroll
+      for (int a1 = 0; a1 < PW; ++a1) {
+        if (a1 < n1) {
+          const T *row = src + ((long long)G2 * Nc[1] + i1[a1]) * Nc[0];
+          T r = T(0);
+#pragma unroll
+          for (int a0 = 0; a0 < PW; ++a0) r += w0[a0] * ld_in<COH>(row + i0[a0]);
+          s += w2 * w1[a1] * r;
+        }
+      }
     }
   }
   return s;
