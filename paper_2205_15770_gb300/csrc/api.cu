@@ -1342,9 +1342,8 @@ static int setup_coarse(stokes_ctx *C) {
   ++C->launches;
   // small matrices: one launch a step, from one buffer into the other (above 1,024 rows every block's own scan of
   // the pivot column would cost more than the pivot kernel)
-  if (nb <= 1024) {
-    double *O = nullptr;
-    if ((st = dalloc(C, &O, (long long)nb * 2 * nb))) return st;
+  double *O = nullptr;
+  if (nb <= 1024 && dalloc(C, &O, (long long)nb * 2 * nb) == STOKES_OK) {
     for (int k = 0; k < nb; ++k) {
       k_gj_step<<<std::min(nb, 304), kVecThreads, 0, C->s>>>(M, O, nb, k, err);
       std::swap(M, O);
@@ -1742,9 +1741,8 @@ static int setup_explicit(stokes_ctx *C) {
   }
   if (le < 1) return STOKES_OK;
   const int n = (int)(C->L32[le].d.n_u + C->L32[le].d.n_p), ldm = (n + 3) / 4 * 4;
-  int st;
   float *M = nullptr;
-  if ((st = dalloc(C, &M, (long long)n * ldm))) return st;
+  if (dalloc(C, &M, (long long)n * ldm) != STOKES_OK) return STOKES_OK;  // no room: the launches stay
   // work vectors of levels 0 .. le for a batch of columns, every column of every vector ld entries apart
   const int cols = std::min(n, kExplicitCols);
   const long long ld = (n + 63) / 64 * 64;
