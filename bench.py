@@ -334,7 +334,7 @@ def traffic_record(key, kernel_src_sha):
 
 def kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("apply.cuh", "apply_col.cuh", "apply_cc.cuh", "common.cuh"):
+    for f in ("apply.cuh", "apply_col.cuh", "apply_cc.cuh", "apply_fx.cuh", "apply_pl.cuh", "common.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2205_15770_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
@@ -348,7 +348,7 @@ NOMINAL_BF16_DENSE_TFLOPS = 2250.0  # GB300 dense bf16 tensor rate (nominal)
 LANES_PER_SM = {32: 128, 64: 2}     # FP32 / FP64 FMA lanes per SM (FP64 = 1/64 of FP32)
 KERNEL_NAMES = {
     "fp32_operator": "full operator K x, FP32, finest level (V-cycle residual and vmult)",
-    "fp64_operator": "full operator K x, FP64, finest level (FGMRES operator; stored per-point geometry)",
+    "fp64_operator": "full operator K x, FP64, finest level (FGMRES operator; stored coefficients)",
     "fp32_a_block": "A block, FP32, finest level (the V-cycle's most frequent application)",
 }
 
@@ -373,6 +373,9 @@ def roofline_entry(key, prec, blocks, avg_ms, n_cells, n_dofs, sm_count, mhz, fm
                   "peak_source": f"derived: {sm_count} SMs x {LANES_PER_SM[prec]} FP{prec} lanes x 2 x {mhz:.0f} MHz",
                   "frac_of_measured_fma": round(ach / fma_tflops, 4),
                   "measured_fma_tflops": round(fma_tflops, 3)})
+        if prec == 64 and shape == 5:
+            e["note"] = ("computed in 64-bit fixed point on the integer units: the FP64 peaks stand for comparison "
+                         "and are not its bound")
         if bf16:
             dv = bf16 * nominal / NOMINAL_BF16_DENSE_TFLOPS
             e["peak_from_measured_bf16"] = round(dv, 4)
