@@ -366,10 +366,10 @@ void stokes_destroy_batch(stokes_batch *batch);
 /* Launch shape of the 3D cell kernel that setup's autotuner chose for `level` and `precision`:
  * 1 or 4 = column kernel with that many warps per CTA, 3 = column kernel with the three velocity
  * components on the three warps of a CTA (shorter per-warp chain for small levels), -1 =
- * point-per-thread kernel, 5 = cell-component kernel (one thread per cell and velocity component,
- * the component's whole tensor in registers; 3D Cartesian levels with k = 2, 3 and FP32 trilinear
- * levels with k = 2, the Laplacian form with a constant rho; other applications on such a level run
- * in the 4-warp column kernel), 0 = not tuned (2D, or STOKES_NO_AUTOTUNE=1).  The environment variable
+ * point-per-thread kernel, 5 = one velocity component of a cell per thread or, split by z plane, per three
+ * threads (k = 2 in FP64: the plane kernel in 64-bit fixed point; k = 2 in FP32: the plane kernel or the
+ * cell-component kernel, whichever setup timed faster; k = 3 Cartesian: the cell-component kernel; the Laplacian
+ * form with a constant rho; other applications on such a level run in the 4-warp column kernel), 0 = not tuned (2D, or STOKES_NO_AUTOTUNE=1).  The environment variable
  * STOKES_TUNING="s32=..;s64=..;f32=..;f64=..[;g32=..]" (comma lists, one value per level, coarsest first)
  * replaces the setup's timings of shapes and smoother forms, e.g. to profile the configuration a
  * plain run chose (a profiler changes the timings); malformed values make setup fail with
@@ -383,14 +383,15 @@ int stokes_get_launch_shape(const stokes_ctx *ctx, int level, int precision, int
  * half of the memory free at setup).  FP32: stored for levels of at most 32^3 cells and read where
  * the setup's timing of the column kernel keeps it (STOKES_TUNING's g32 list otherwise; 0 without
  * autotuning), released at setup where it is not kept; STOKES_GEO=none stores neither precision.
- * The cell-component kernel (shape 5) evaluates the FP32 geometry itself either way.  The geometry
+ * The cell-component kernel (shape 5) evaluates the FP32 geometry itself either way; the plane kernels read
+ * coefficients of their own, not reported here.  The geometry
  * is that of the cells' bi/trilinear maps T_tau (Sec. 2) at the Gauss points.  HOST output;
  * STOKES_EINVAL for a level out of range or a precision other than 32 / 64. */
 int stokes_get_geometry_stored(const stokes_ctx *ctx, int level, int precision, int *stored);
 
-/* 1 if smoothing on `level` / `precision` runs in the fused form (k_A = 1, 3D, column kernel: the
+/* 1 if smoothing on `level` / `precision` runs in the fused form (k_A = 1; the
  * Chebyshev-Jacobi and Uzawa vector updates of Sec. 3.3.1 evaluated inside the cell-kernel
- * gathers, 5 + 3 k_S launches per step), 0 if in the unfused form (separate vector kernels).
+ * gathers, 5 + 3 k_S launches per step, 5 + k_S with the explicit S~), 0 if in the unfused form (separate vector kernels).
  * Setup times both forms per level and keeps the faster (STOKES_NO_AUTOTUNE=1: fused wherever
  * eligible; STOKES_NO_FUSE=1: never).  Level 0 (direct solve) reports 0.  HOST output. */
 int stokes_get_smoother_fusion(stokes_ctx *ctx, int level, int precision, int *fused);
