@@ -60,6 +60,7 @@ __device__ __forceinline__ T restrict_terms(const LevelDesc<T> &F, const LevelDe
   const T *ssrc = SUB ? minus + off : nullptr;
   const Xfer1D<T> &ax = X.r[sp][0], &ay = X.r[sp][1], &az = X.r[sp][2];
   const int n0 = ax.cnt[G0], n1 = ay.cnt[G1], n2 = az.cnt[G2];
+  if (n0 == 0 || n1 == 0 || n2 == 0) return T(0);  // a node on a Dirichlet face (t0 is divided by n1 below)
   int f0[W];
   T w0[W];
 #pragma unroll
