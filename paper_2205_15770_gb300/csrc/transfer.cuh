@@ -146,7 +146,7 @@ __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDes
   T w0[PW], w1[PW];
 #pragma unroll
   for (int a = 0; a < PW; ++a) {
-    i0[a] = ax.idx[g0 * W + (a < n0 ? a : 0)];  // past the row: its first node again, with weight 0
+    i0[a] = a < n0 ? ax.idx[g0 * W + a] : 0;
     w0[a] = a < n0 ? ax.w[g0 * W + a] : T(0);
     i1[a] = a < n1 ? ay.idx[g1 * W + a] : 0;
     w1[a] = a < n1 ? ay.w[g1 * W + a] : T(0);
@@ -163,7 +163,8 @@ __device__ __forceinline__ T prolong_entry(const LevelDesc<T> &F, const LevelDes
           const T *row = src + ((long long)G2 * Nc[1] + i1[a1]) * Nc[0];
           T r = T(0);
 #pragma unroll
-          for (int a0 = 0; a0 < PW; ++a0) r += w0[a0] * ld_in<COH>(row + i0[a0]);
+          for (int a0 = 0; a0 < PW; ++a0)
+            if (a0 < n0) r += w0[a0] * ld_in<COH>(row + i0[a0]);
           s += w2 * w1[a1] * r;
         }
       }

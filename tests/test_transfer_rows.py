@@ -1,5 +1,6 @@
 """The row functions of the grid transfers, compiled for the host (no GPU): every coarse and fine DoF of a small 2D and 3D
-pair against plain nested sums, with empty 1D rows (nodes on Dirichlet faces) along every axis."""
+pair against plain nested sums, with empty 1D rows (nodes on Dirichlet faces) along every axis,
+and with an infinity or NaN among the inputs (it reaches the sums it belongs to, as itself, and no others)."""
 import subprocess
 
 import pytest
@@ -37,13 +38,13 @@ static Rows rows(int n, int nodes, int most, int W, bool fixed) {
     r.cnt[i] = 1 + (int)(rng() % std::min(most, nodes));
     for (int a = 0; a < r.cnt[i]; ++a) {
       r.idx[i * W + a] = (int)((rng() % 2 + 2 * a) % nodes);
-      r.w[i * W + a] = (rng() % 2000) / 1000.0 - 1.0;
+      r.w[i * W + a] = (rng() % 2000) / 1000.0 - 0.9995;  // never zero
     }
   }
   return r;
 }
 template <int W>
-static int check(int dim, int k, const int *nc, unsigned fixed_axes) {
+static int check(int dim, int k, const int *nc, unsigned fixed_axes, double planted = 0.5) {
   LevelDesc<double> L[2]{};  // coarse, fine
   for (int f = 0; f < 2; ++f) {
     L[f].dim = dim;
@@ -73,6 +74,7 @@ static int check(int dim, int k, const int *nc, unsigned fixed_axes) {
     std::vector<double> in(from.n_u + from.n_p), sub(in.size());
     for (double &v : in) v = (rng() % 2000) / 1000.0 - 1.0;
     for (double &v : sub) v = (rng() % 2000) / 1000.0 - 1.0;
+    for (int c = 0; c <= dim; ++c) in[c < dim ? c * from.nv + from.nv / 2 : from.n_u + from.n_p / 2] = planted;
     for (long long i = 0; i < to.n_u + to.n_p; ++i) {
       const int sp = i < to.n_u ? 0 : 1;
       const int *N = sp ? to.Pn : to.N, *M = sp ? from.Pn : from.N;
@@ -98,7 +100,11 @@ static int check(int dim, int k, const int *nc, unsigned fixed_axes) {
         r[0] = prolong_entry<double, W>(to, from, X, in.data(), i);
       }
       // at most 17^3 terms of at most 2, three products each: 4,913 x 2 x 8 roundings
-      for (int q = 0; q < 3; ++q) bad += !(std::fabs(r[q] - s[q > 0]) <= 4913 * 2 * 8 * 0x1p-53);
+      for (int q = 0; q < (d ? 1 : 3); ++q) {
+        const double e = s[q > 0];
+        bad += std::isfinite(e) ? !(std::fabs(r[q] - e) <= 4913 * 2 * 8 * 0x1p-53)
+                                : std::isnan(r[q]) != std::isnan(e) || (!std::isnan(e) && r[q] != e);
+      }
     }
   }
   if (bad) std::printf("dim %d k %d axes %u: %d rows off\n", dim, k, fixed_axes, bad);
@@ -110,6 +116,7 @@ int main() {
   for (unsigned axes = 0; axes < 8; ++axes) {
     if (axes < 4) bad += check<9>(2, 2, n2, axes) + check<13>(2, 3, n2, axes) + check<17>(2, 4, n2, axes);
     bad += check<9>(3, 2, n3, axes) + check<13>(3, 3, n3, axes);
+    for (double v : {(double)INFINITY, -(double)INFINITY, (double)NAN}) bad += check<9>(3, 2, n3, axes, v) + check<13>(3, 3, n3, axes, v);
   }
   return bad ? 1 : 0;
 }
