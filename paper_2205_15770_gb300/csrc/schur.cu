@@ -57,6 +57,17 @@ __global__ void __launch_bounds__(32 * kStencilW)
   for (int l = 0; l < LINES; ++l)
 #pragma unroll
     for (int j = 0; j < W; ++j) s += a[l * W + j] * xs[w][l][lane + j];
+  if (!isfinite(s)) {  // zero times an infinity or NaN is not nothing: leave out what lies off the grid
+    const int r = row / P0, gx = row - r * P0, gy = r % P1, gz = r / P1, P2 = n / (P0 * P1);
+    s = T(0);
+    for (int l = 0; l < LINES; ++l) {
+      const int y = gy + (DIM == 3 ? l : w) - R, z = DIM == 3 ? gz + w - R : 0;
+      for (int j = 0; j < W; ++j) {
+        const int x = gx + j - R;
+        if (x >= 0 && x < P0 && y >= 0 && y < P1 && z >= 0 && z < P2) s += m[(l * W + j) * ldm] * xs[w][l][lane + j];
+      }
+    }
+  }
   part[w][lane] = s;
   __syncthreads();
   if (w != 0 || row >= n) return;
