@@ -140,9 +140,24 @@ __global__ void k_coarse_apply(const double *__restrict__ Kinv, int n0, const T 
 
 // ---- explicit cycle of a small level (setup_explicit) --------------------------------------------
 // x = M b, M n x n with rows of ldm entries (16-byte multiples, the padding zero): one warp per row, every
-// 16-byte piece of the row in flight.  Bound by the matrix read from L2: 2,312 rows (21 MB)
-// take 5 us, 2,467 rows 5.8 us.
+// 16-byte piece of the row in flight.  Bound by the matrix read from L2 and a launch's latencies.  The coarse solve
+// inside M had its sums in FP64, so the sums here carry their rounding errors along (the error-free sum and product of
+// Knuth and Dekker, "dot2"): plain FP32 sums left up to 1.2 times the error of the launches that M replaces, these
+// 0.7-0.9 of it (cycle without smoothing, seven hierarchies), for 2.4 us more with 2,467 rows (24 MB; 5.8 us plain) and
+// 3.6 with 2,312 (5 us).
 constexpr int kExplicitWarps = 16;
+struct Sum2 {  // s + e
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float p, float pe) {
+    const float t = s + p, z = t - s;
+    e += ((s - (t - z)) + (p - z)) + pe;
+    s = t;
+  }
+  __device__ __forceinline__ void add_product(float a, float b) {
+    const float p = __fmul_rn(a, b);  // (not to be contracted into the addition)
+    add(p, fmaf(a, b, -p));
+  }
+};
 __global__ void __launch_bounds__(32 * kExplicitWarps)
     k_explicit_apply(const float *__restrict__ M, int n, int ldm, const float *__restrict__ b, float *__restrict__ x) {
   pdl_enter();
@@ -150,20 +165,22 @@ __global__ void __launch_bounds__(32 * kExplicitWarps)
   if (row >= n) return;
   const float4 *m = reinterpret_cast<const float4 *>(M + (long long)row * ldm), *v = reinterpret_cast<const float4 *>(b);
   const int full = n / 4;
-  float s[4] = {};
+  Sum2 s[4];
 #pragma unroll 8
   for (int j = lane; j < full; j += 32) {
     const float4 a = __ldg(m + j), c = v[j];
-    s[0] += a.x * c.x;
-    s[1] += a.y * c.y;
-    s[2] += a.z * c.z;
-    s[3] += a.w * c.w;
+    s[0].add_product(a.x, c.x);
+    s[1].add_product(a.y, c.y);
+    s[2].add_product(a.z, c.z);
+    s[3].add_product(a.w, c.w);
   }
-  float t = (s[0] + s[1]) + (s[2] + s[3]);
   const int j = 4 * full + lane;
-  if (j < n) t += M[(long long)row * ldm + j] * b[j];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-  if (lane == 0) x[row] = t;
+  if (j < n) s[0].add_product(M[(long long)row * ldm + j], b[j]);
+  s[0].add(s[1].s, s[1].e);
+  s[2].add(s[3].s, s[3].e);
+  s[0].add(s[2].s, s[2].e);
+  for (int o = 16; o > 0; o >>= 1) s[0].add(__shfl_down_sync(0xffffffffu, s[0].s, o), __shfl_down_sync(0xffffffffu, s[0].e, o));
+  if (lane == 0) x[row] = s[0].s + s[0].e;
 }
 // unit vectors j0 + column of length n
 __global__ void k_unit_cols(float *b, int n, int j0, long long ld) {
@@ -1727,7 +1744,10 @@ static int setup_schur(stokes_ctx *C) {
 // most kExplicitBytes becomes explicit (FP32 multigrid, C = 0, not in deterministic mode: M is summed by
 // atomics).  The line: a matrix of 48 MB, 3,464 unknowns, is read in 6 us and built in about 10 ms; at twice
 // the unknowns (6^3 cells: 192 MB, beyond L2) the build is four times as long and the read 30 us.
-// M's columns are the cycle of the unit vectors, kExplicitCols of them in every launch (column()).
+// M's columns are the cycle of the unit vectors, kExplicitCols of them in every launch (column()), by kernels as exact as
+// the launches': with the 2D cells in the point kernel the whole FP32 cycle was 1.03 (box) to 1.06 (warped, at most 1.19)
+// times as far from the FP64 cycle as by launches, with the 2D kernel 1.00 (means of 14 meshes; 3D 1.00), and
+// the 2D matrix of 2,467 rows takes 4.1 ms instead of 6.8.
 // STOKES_NO_EXPLICIT=1 keeps the launches.
 constexpr long long kExplicitBytes = 48ll << 20;
 constexpr int kExplicitCols = 512;

@@ -79,8 +79,14 @@ struct Line {
 template <int K, typename T, int MODE, bool CART, bool FUSED>
 __global__ void __launch_bounds__(64)
     stokes_cell_apply_2d(const LevelDesc<T> L, const T *__restrict__ u, const T *__restrict__ p, T *__restrict__ yu,
-                         T *__restrict__ yp, const Fuse<T> F) {
+                         T *__restrict__ yp, const Fuse<T> F, const long long ld) {
   pdl_enter();
+  if constexpr (!FUSED) {
+    u = column(u, ld);
+    p = column(p, ld);
+    yu = column(yu, ld);
+    yp = column(yp, ld);
+  }
   constexpr int N = K + 1, NP = K;
   constexpr bool DO_A = MODE & kApplyA, DO_BT = MODE & kApplyBT, DO_B = MODE & kApplyB;
   constexpr bool NEED_U = DO_A || DO_B;
@@ -336,24 +342,26 @@ __global__ void __launch_bounds__(64)
 }
 
 template <int K, typename T, int MODE, bool FUSED>
-static int launch_2d_mode(const LevelDesc<T> &L, const T *u, const T *p, T *yu, T *yp, cudaStream_t s, const Fuse<T> &F) {
-  const dim3 grid((unsigned)((L.n_cells + 31) / 32)), block(64);
+static int launch_2d_mode(const LevelDesc<T> &L, const T *u, const T *p, T *yu, T *yp, cudaStream_t s, const Fuse<T> &F,
+                          int cols, long long ld) {
+  const dim3 grid((unsigned)((L.n_cells + 31) / 32), (unsigned)cols), block(64);
   if (L.cartesian)
-    launch_kernel(stokes_cell_apply_2d<K, T, MODE, true, FUSED>, grid, block, 0, s, L, u, p, yu, yp, F);
+    launch_kernel(stokes_cell_apply_2d<K, T, MODE, true, FUSED>, grid, block, 0, s, L, u, p, yu, yp, F, ld);
   else
-    launch_kernel(stokes_cell_apply_2d<K, T, MODE, false, FUSED>, grid, block, 0, s, L, u, p, yu, yp, F);
+    launch_kernel(stokes_cell_apply_2d<K, T, MODE, false, FUSED>, grid, block, 0, s, L, u, p, yu, yp, F, ld);
   return 0;
 }
-// A, B^T, B, A + B^T and the full operator; -1 for other modes (mass, symmetric form, unmasked lifting).
+// A, B^T, B, A + B^T and the full operator; -1 for other modes (mass, symmetric form, unmasked lifting).  cols: plain
+// launches on that many vectors at once, ld entries apart.
 template <int K, typename T, bool FUSED>
 static int launch_2d(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp, cudaStream_t s,
-                     const Fuse<T> &F) {
+                     const Fuse<T> &F, int cols = 1, long long ld = 0) {
   switch (mode) {
-    case kApplyA: return launch_2d_mode<K, T, kApplyA, FUSED>(L, u, p, yu, yp, s, F);
-    case kApplyBT: return launch_2d_mode<K, T, kApplyBT, FUSED>(L, u, p, yu, yp, s, F);
-    case kApplyB: return launch_2d_mode<K, T, kApplyB, FUSED>(L, u, p, yu, yp, s, F);
-    case kApplyA | kApplyBT: return launch_2d_mode<K, T, kApplyA | kApplyBT, FUSED>(L, u, p, yu, yp, s, F);
-    case kApplyA | kApplyBT | kApplyB: return launch_2d_mode<K, T, kApplyA | kApplyBT | kApplyB, FUSED>(L, u, p, yu, yp, s, F);
+    case kApplyA: return launch_2d_mode<K, T, kApplyA, FUSED>(L, u, p, yu, yp, s, F, cols, ld);
+    case kApplyBT: return launch_2d_mode<K, T, kApplyBT, FUSED>(L, u, p, yu, yp, s, F, cols, ld);
+    case kApplyB: return launch_2d_mode<K, T, kApplyB, FUSED>(L, u, p, yu, yp, s, F, cols, ld);
+    case kApplyA | kApplyBT: return launch_2d_mode<K, T, kApplyA | kApplyBT, FUSED>(L, u, p, yu, yp, s, F, cols, ld);
+    case kApplyA | kApplyBT | kApplyB: return launch_2d_mode<K, T, kApplyA | kApplyBT | kApplyB, FUSED>(L, u, p, yu, yp, s, F, cols, ld);
     default: return -1;
   }
 }

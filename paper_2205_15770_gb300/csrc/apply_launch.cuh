@@ -90,10 +90,12 @@ int launch_cell_apply_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, co
                      : launch_apply_dim<2, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho);
 }
 
-// The same applications on `cols` vectors at once, ld entries apart, in the point kernel.
+// The same applications on `cols` vectors at once, ld entries apart, in the 2D kernel where it serves them, else in the
+// point kernel.
 template <int K, typename T>
 int launch_cell_apply_cols_k(const LevelDesc<T> &L, const Tab1D<T> *tab, int mode, const T *u, const T *p, T *yu, T *yp,
                              cudaStream_t s, const T *rho, int cols, long long ld) {
+  if (L.dim == 2 && !rho && launch_2d<K, T, false>(L, mode, u, p, yu, yp, s, Fuse<T>{}, cols, ld) == 0) return 0;
   if (L.dim == 3)
     return L.cartesian ? launch_apply_dim<3, K, T, true>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld)
                        : launch_apply_dim<3, K, T, false>(L, tab, mode, u, p, yu, yp, s, rho, cols, ld);
