@@ -342,6 +342,8 @@ struct stokes_ctx {
   int pq_member = 0;
   bool use_graphs = true;
   bool fuse = true;  // fused smoothing where eligible (STOKES_NO_FUSE=1: the unfused path)
+  // the plane kernels' coefficient tables: not wanted (lean: a setup that ran out of memory with them), stored (tables)
+  bool lean = false, tables = false;
   std::vector<Tuned> tuned64, tuned32;  // the setup's choices per level (empty: not timed)
   GraphSlot g32[2], g64[2];  // [x_zero]
   // FP32 cycle of level le from a zero start as an explicit matrix (setup_explicit; -1: none)
@@ -2088,18 +2090,24 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
         if ((st = dalloc(C, &geo_l, cells * per))) return st;
         launch_col_geometry<double>(d, geo_l, C->s);
         SMF_CUDA_OK(cudaGetLastError());
-        if (k == 2 && gbytes <= (long long)(free_b / 4)) {
-          if ((st = dalloc(C, &geox_l, fx_geometry_bytes(cells) / (long long)sizeof(double)))) return st;
-          launch_fx_geometry(d, geox_l, C->s);
-          SMF_CUDA_OK(cudaGetLastError());
-        }
       }
-      // coefficients of the FP32 plane kernel (2,304 B a cell), the same budget
+      // Coefficients of the plane kernels (k = 2, not in deterministic mode): 3,694 bytes a cell in FP64 beside the
+      // geometry, 2,304 in FP32.  Without them the column and cell-component kernels serve the level, so each is stored
+      // only while it leaves three quarters of the memory that is free by then.
+      const auto room = [&](long long bytes) {
+        size_t f = 0, t = 0;
+        return k == 2 && !C->det && !C->lean && cudaMemGetInfo(&f, &t) == cudaSuccess && bytes <= (long long)(f / 4);
+      };
+      const long long xbytes = fx_geometry_bytes(cells), pbytes = pl_geometry_bytes(cells);
+      if (geo_l && room(xbytes) && dalloc(C, &geox_l, xbytes / (long long)sizeof(double)) == STOKES_OK) {
+        C->tables = true;
+        launch_fx_geometry(d, geox_l, C->s);
+        SMF_CUDA_OK(cudaGetLastError());
+      }
       const char *np = getenv("STOKES_NO_PLANE");
-      const long long pbytes = pl_geometry_bytes(cells);
-      if (g64 && k == 2 && !C->det && !(np && np[0] == '1') && pbytes <= (long long)(total_b / 16) &&
-          pbytes <= (long long)(free_b / 4)) {
-        if ((st = dalloc(C, &geop_l, pbytes / (long long)sizeof(float)))) return st;
+      if (g64 && !(np && np[0] == '1') && pbytes <= (long long)(total_b / 16) && room(pbytes) &&
+          dalloc(C, &geop_l, pbytes / (long long)sizeof(float)) == STOKES_OK) {
+        C->tables = true;
         launch_pl_geometry(d, geop_l, C->s);
         SMF_CUDA_OK(cudaGetLastError());
       }
@@ -3453,25 +3461,31 @@ static int setup_like(const stokes_mesh *mesh, int k, double mu, double gamma_rh
     const int sa = noalloc_scratch_address(&scratch);
     if (sa != STOKES_OK) return sa;
   }
-  stokes_ctx *C = new (std::nothrow) stokes_ctx();
-  if (!C) {
-    set_error("host allocation failed");
-    return STOKES_ENOMEM;
-  }
-  cudaStream_t user = (cudaStream_t)stream;
-  cudaStreamSynchronize(user);
-  if (cudaGetDevice(&C->device) != cudaSuccess) {
-    cudaGetLastError();
-    C->device = -1;
-  }
-  int st = do_setup(mesh, k, mu, gamma_rho, mu_cell, opts, like, C);
-  if (st == STOKES_OK) {
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) st = cuda_fail(e, "setup kernels", __FILE__, __LINE__);
-  }
-  if (st != STOKES_OK) {
+  cudaStreamSynchronize((cudaStream_t)stream);
+  stokes_ctx *C = nullptr;
+  int st = STOKES_OK;
+  // the tables are stored before the vectors that a context cannot do without: a setup that runs out of memory with
+  // them starts again without them
+  for (bool lean = false;; lean = true) {
+    C = new (std::nothrow) stokes_ctx();
+    if (!C) {
+      set_error("host allocation failed");
+      return STOKES_ENOMEM;
+    }
+    if (cudaGetDevice(&C->device) != cudaSuccess) {
+      cudaGetLastError();
+      C->device = -1;
+    }
+    C->lean = lean;
+    st = do_setup(mesh, k, mu, gamma_rho, mu_cell, opts, like, C);
+    if (st == STOKES_OK) {
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) st = cuda_fail(e, "setup kernels", __FILE__, __LINE__);
+    }
+    if (st == STOKES_OK) break;
+    const bool again = st == STOKES_ENOMEM && C->tables;
     stokes_destroy(C);
-    return st;
+    if (!again) return st;
   }
   *out = C;
   return STOKES_OK;
