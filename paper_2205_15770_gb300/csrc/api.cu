@@ -1329,6 +1329,8 @@ static int setup_coarse(stokes_ctx *C) {
   double *K0 = nullptr, *e = nullptr, *M = nullptr, *fac = nullptr;
   int *err = nullptr;
   int st;
+  if ((st = dalloc(C, &C->Kinv, n0 * n0))) return st;
+  const size_t kept = C->allocs.size();  // what follows is work of this function
   if ((st = dalloc(C, &K0, n0 * n0))) return st;
   if ((st = dalloc(C, &e, n0))) return st;
   const int bord = C->pker ? 1 : 0;
@@ -1336,7 +1338,6 @@ static int setup_coarse(stokes_ctx *C) {
   if ((st = dalloc(C, &M, (long long)nb * 2 * nb))) return st;
   if ((st = dalloc(C, &fac, nb))) return st;
   if ((st = dalloc(C, &err, 1))) return st;
-  if ((st = dalloc(C, &C->Kinv, n0 * n0))) return st;
   if (!C->det && !R.hasC()) {
     // every column in one launch of the point kernel (the unit vectors lie in M, which is written afterwards), and the
     // identity rows of constrained DoFs; one at a time this took three launches a column
@@ -1381,6 +1382,10 @@ static int setup_coarse(stokes_ctx *C) {
   int herr = 0;
   SMF_CUDA_OK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, C->s));
   SMF_CUDA_OK(cudaStreamSynchronize(C->s));
+  while (C->allocs.size() > kept) {
+    cudaFree(C->allocs.back());
+    C->allocs.pop_back();
+  }
   if (herr) {
     set_error("coarse matrix is singular");
     return STOKES_EBREAKDOWN;
