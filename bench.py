@@ -78,7 +78,7 @@ def tuning_string(S):
     timings taken under a profiler choose differently)."""
     j = lambda v: ",".join(str(int(x)) for x in v)
     return (f"s32={j(S.launch_shapes(32))};s64={j(S.launch_shapes(64))};f32={j(S.fused_levels(32))};"
-            f"f64={j(S.fused_levels(64))};g32={j(S.geometry_stored(32))}")
+            f"f64={j(S.fused_levels(64))};g32={j(S.geometry_stored(32))};p32={j(S.plane_levels(32))}")
 
 
 # ---------------------------------------------------------------------------------------------

@@ -29,7 +29,7 @@
  * arithmetic, so none changes a result beyond rounding order):
  *  - STOKES_NO_AUTOTUNE=1: no setup timing; default launch shapes, fused smoothing where eligible,
  *    per-point geometry evaluated by the FP32 kernels.
- *  - STOKES_TUNING="s32=..;s64=..;f32=..;f64=..[;g32=..]": the setup's choices pinned (see
+ *  - STOKES_TUNING="s32=..;s64=..;f32=..;f64=..[;g32=..][;p32=..]": the setup's choices pinned (see
  *    stokes_get_launch_shape).
  *  - STOKES_NO_FUSE=1: unfused smoothing everywhere.  STOKES_NO_GRAPHS=1: no CUDA-graph capture.
  *  - STOKES_HOST_KRYLOV=1: the FGMRES iterations driven from the host (stokes_krylov_mode).
@@ -369,8 +369,9 @@ void stokes_destroy_batch(stokes_batch *batch);
  * point-per-thread kernel, 5 = one velocity component of a cell per thread or, split by z plane, per three
  * threads (k = 2 in FP64: the plane kernel in 64-bit fixed point; k = 2 in FP32: the plane kernel or the
  * cell-component kernel, whichever setup timed faster; k = 3 Cartesian: the cell-component kernel; the Laplacian
- * form with a constant rho; other applications on such a level run in the 4-warp column kernel), 0 = not tuned (2D, or STOKES_NO_AUTOTUNE=1).  The environment variable
- * STOKES_TUNING="s32=..;s64=..;f32=..;f64=..[;g32=..]" (comma lists, one value per level, coarsest first)
+ * form with a constant rho; other applications on such a level run in the 4-warp column kernel), 0 = not tuned
+ * (2D, or STOKES_NO_AUTOTUNE=1).  The environment variable
+ * STOKES_TUNING="s32=..;s64=..;f32=..;f64=..[;g32=..][;p32=..]" (comma lists, one value per level, coarsest first)
  * replaces the setup's timings of shapes and smoother forms, e.g. to profile the configuration a
  * plain run chose (a profiler changes the timings); malformed values make setup fail with
  * STOKES_EINVAL.  HOST output.  No counterpart in the paper (a launch choice of this library). */
@@ -388,6 +389,13 @@ int stokes_get_launch_shape(const stokes_ctx *ctx, int level, int precision, int
  * is that of the cells' bi/trilinear maps T_tau (Sec. 2) at the Gauss points.  HOST output;
  * STOKES_EINVAL for a level out of range or a precision other than 32 / 64. */
 int stokes_get_geometry_stored(const stokes_ctx *ctx, int level, int precision, int *stored);
+
+/* 1 if launch shape 5 on `level` in `precision` (32 or 64) is a plane kernel (k = 2: a z plane of a cell's component
+ * per thread), 0 if it is the cell-component kernel.  FP64: the plane kernel wherever its coefficients are stored or
+ * the level is Cartesian.  FP32: the one that setup timed faster, or STOKES_TUNING's p32 list (1 on a level without
+ * the plane kernel makes setup fail with STOKES_EINVAL; without the list, the plane kernel where the level has it).
+ * HOST output; STOKES_EINVAL for a level out of range or a precision other than 32 / 64.  No counterpart in the paper. */
+int stokes_get_plane_form(const stokes_ctx *ctx, int level, int precision, int *plane);
 
 /* 1 if smoothing on `level` / `precision` runs in the fused form (k_A = 1; the
  * Chebyshev-Jacobi and Uzawa vector updates of Sec. 3.3.1 evaluated inside the cell-kernel

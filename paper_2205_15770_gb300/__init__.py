@@ -417,6 +417,16 @@ class StokesMG:
             out.append(bool(v.value))
         return out
 
+    def plane_levels(self, precision=32):
+        """Per level: True where launch shape 5 is a plane kernel, False where it is the cell-component kernel
+        (stokes_get_plane_form)."""
+        out = []
+        for l in range(self.n_levels):
+            v = C.c_int()
+            self._check(self._lib.stokes_get_plane_form(self._ctx, l, precision, C.byref(v)))
+            out.append(bool(v.value))
+        return out
+
     def fused_levels(self, precision=32):
         """Per level: True where smoothing runs in the fused form (stokes_get_smoother_fusion)."""
         out = []

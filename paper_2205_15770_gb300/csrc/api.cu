@@ -1809,16 +1809,19 @@ static int setup_explicit(stokes_ctx *C) {
   return STOKES_OK;
 }
 
-// STOKES_TUNING="s32=a,b,..;s64=..;f32=..;f64=..[;g32=..]" replaces the setup's timings: launch
+// STOKES_TUNING="s32=a,b,..;s64=..;f32=..;f64=..[;g32=..][;p32=..]" replaces the setup's timings: launch
 // shapes (1, 3, 4, -1 or 5) and smoother forms (1 fused, 0 unfused) per level, coarsest first, for
 // FP32 and FP64, and optionally whether the FP32 column kernels read the stored per-point geometry
-// (1) or evaluate it (0, the default).  Timings taken under a profiler differ from plain runs; a
+// (1) or evaluate it (0, the default) and whether FP32 shape 5 is the plane kernel (1, the default where the level has
+// it) or the cell-component kernel (0).  Timings taken under a profiler differ from plain runs; a
 // profile of the configuration that a plain run chose passes that run's choices here
-// (stokes_get_launch_shape, stokes_get_smoother_fusion and stokes_get_geometry_stored read them).
-static int parse_tuning(const char *spec, int nl, std::vector<int> tune[5]) {
-  const char *keys[5] = {"s32=", "s64=", "f32=", "f64=", "g32="};
-  for (int t = 0; t < 5; ++t) {
+// (stokes_get_launch_shape, stokes_get_smoother_fusion, stokes_get_geometry_stored and stokes_get_plane_form read them).
+constexpr int kTuneLists = 6;
+static int parse_tuning(const char *spec, int nl, std::vector<int> tune[kTuneLists]) {
+  const char *keys[kTuneLists] = {"s32=", "s64=", "f32=", "f64=", "g32=", "p32="};
+  for (int t = 0; t < kTuneLists; ++t) {
     const char *p = std::strstr(spec, keys[t]);
+    if (!p && t == 5) continue;  // empty: as the level has it
     if (!p && t == 4) {
       tune[t].assign(nl, 0);
       continue;
@@ -2203,7 +2206,7 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
 
   // launch-shape autotuning (STOKES_NO_AUTOTUNE=1 keeps the default shape; STOKES_TUNING fixes
   // shapes and smoother forms instead, see parse_tuning)
-  std::vector<int> tune[5];
+  std::vector<int> tune[kTuneLists];
   const bool pinned = getenv("STOKES_TUNING") != nullptr && !C->det;
   if (pinned && (st = parse_tuning(getenv("STOKES_TUNING"), nl, tune))) return st;
   if (pinned) {
@@ -2217,6 +2220,13 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
           return STOKES_EINVAL;
         }
         C->L32[l].geo = tune[4][l] ? C->L32[l].geo_stored : nullptr;
+        if (!tune[5].empty()) {
+          if (tune[5][l] && !C->L32[l].plane) {
+            set_error("STOKES_TUNING: p32 asks for the plane kernel on level " + std::to_string(l) + ", which has none (3D, k = 2)");
+            return STOKES_EINVAL;
+          }
+          C->L32[l].plane = tune[5][l] != 0;
+        }
       }
     }
   }
@@ -4102,6 +4112,16 @@ int stokes_get_geometry_stored(const stokes_ctx *C, int level, int precision, in
     return STOKES_EINVAL;
   }
   *stored = (precision == 64 ? C->L64[level].geo != nullptr : C->L32[level].geo != nullptr) ? 1 : 0;
+  return STOKES_OK;
+}
+
+int stokes_get_plane_form(const stokes_ctx *C, int level, int precision, int *plane) {
+  if (!C || level < 0 || level >= C->nl || !plane || (precision != 32 && precision != 64)) {
+    set_error("invalid stokes_get_plane_form arguments");
+    return STOKES_EINVAL;
+  }
+  const LevelDesc<double> &d = C->L64[level].d;
+  *plane = precision == 32 ? C->L32[level].plane : d.dim == 3 && d.k == 2 && !C->det && (d.cartesian || C->L64[level].geox);
   return STOKES_OK;
 }
 
