@@ -1747,10 +1747,10 @@ static int setup_schur(stokes_ctx *C) {
 // The FP32 cycle of a small level below the finest as an explicit matrix.  From a zero start the gamma
 // recursive calls are linear in the right-hand side, x_l = M b_l, and on a small level their ~40 (2D: per
 // level) dependent launches of 2-4 us cost far more than reading M: 4^3 and the 2^3 coarse solve 130-156 us
-// against 5 us for M's 21 MB, which stay in L2; three 2D levels up to 16^2 460 us against 6.  So the largest level l <= n_levels - 2 whose M takes at
-// most kExplicitBytes becomes explicit (FP32 multigrid, C = 0, not in deterministic mode: M is summed by
-// atomics).  The line: a matrix of 48 MB, 3,464 unknowns, is read in 6 us and built in about 10 ms; at twice
-// the unknowns (6^3 cells: 192 MB, beyond L2) the build is four times as long and the read 30 us.
+// against 8.6 us for M's 21 MB, which stay in L2; three 2D levels up to 16^2 460 us against 8.2.  So the largest level
+// l <= n_levels - 2 whose M takes at most kExplicitBytes becomes explicit (FP32 multigrid, C = 0, not in deterministic
+// mode: M is summed by atomics).  The line: a matrix of 48 MB, 3,464 unknowns, stays in L2 and is built in about 10 ms;
+// at twice the unknowns (6^3 cells: 192 MB, beyond L2) the build is four times as long and the read 30 us.
 // M's columns are the cycle of the unit vectors, kExplicitCols of them in every launch (column()), by kernels as exact as
 // the launches': with the 2D cells in the point kernel the whole FP32 cycle was 1.03 (box) to 1.06 (warped, at most 1.19)
 // times as far from the FP64 cycle as by launches, with the 2D kernel 1.00 (means of 14 meshes; 3D 1.00), and
@@ -2231,7 +2231,9 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
     }
   }
   // (a change of viscosities takes over the choices of the context it replaces: the same mesh, degree and forms; timing
-  // them again: gradient 16^3, which is one change and two solves, 55 -> 82 ms)
+  // them again: gradient 16^3, which is one change and two solves, 55 -> 82 ms.  The smoother forms were timed with the
+  // explicit S~, which a change does not build: of 62 levels (2D 128^2, 8^3 to 32^3, k_S 1 to 3, both precisions) the
+  // form kept was the faster one without S~ too, or within 3 %)
   bool timed = false, taken = false;
   {
     const char *na = getenv("STOKES_NO_AUTOTUNE");
@@ -2342,7 +2344,9 @@ static int do_setup(const stokes_mesh *mesh, int k, double mu, double gamma_rho,
     if ((st = zero_level_work(C, C->L64[l]))) return st;
     if ((st = zero_level_work(C, C->L32[l]))) return st;
   }
-  if (!like) {  // (for a change of viscosities the matrices would cost what its few solves gain)
+  // (for a change of viscosities the matrices cost what 30 FP64 or 100 FP32 cycles gain: 8.5 ms at 16^3, 280 and 80 us a
+  // cycle; 19 ms at 32^3 FP32, 163 us)
+  if (!like) {
     if ((st = setup_schur<float>(C))) return st;
     if ((st = setup_schur<double>(C))) return st;
   }

@@ -1096,8 +1096,7 @@ int launch_cell_apply_cc_k(const LevelDesc<T> &L, int mode, const T *u, const T 
 template <int K, typename T>
 int launch_cell_apply_cc_fused_k(const LevelDesc<T> &L, int mode, const T *u, const T *p, T *yu, T *yp,
                                  const T *geo, const Fuse<T> &F, cudaStream_t s) {
-  {
-    if (L.k != 2 || !cc_serves(L, geo)) return -1;
+  if (L.k != 2 || !cc_serves(L, geo)) return -1;
 #define SMF_CCF_CASE(M)                                                                                         \
   case M: {                                                                                                     \
     using CL = CcLaunch<2, T, M, false>;                                                                        \
@@ -1112,16 +1111,15 @@ int launch_cell_apply_cc_fused_k(const LevelDesc<T> &L, int mode, const T *u, co
                     L, u, p, yu, yp, geo, F);                                                                   \
     return 0;                                                                                                   \
   }
-    switch (mode) {
-      SMF_CCF_CASE(kApplyA)
-      SMF_CCF_CASE(kApplyBT)
-      SMF_CCF_CASE(kApplyB)
-      SMF_CCF_CASE(kApplyA | kApplyBT)
-      SMF_CCF_CASE(kApplyA | kApplyBT | kApplyB)
-      default: return -1;
-    }
-#undef SMF_CCF_CASE
+  switch (mode) {
+    SMF_CCF_CASE(kApplyA)
+    SMF_CCF_CASE(kApplyBT)
+    SMF_CCF_CASE(kApplyB)
+    SMF_CCF_CASE(kApplyA | kApplyBT)
+    SMF_CCF_CASE(kApplyA | kApplyBT | kApplyB)
+    default: return -1;
   }
+#undef SMF_CCF_CASE
 }
 
 }  // namespace smf

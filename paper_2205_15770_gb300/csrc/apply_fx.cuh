@@ -28,9 +28,10 @@
 // 2^58.8 (rows of G, 2^62), each of B^T's 2^57 (pressure integers 2^59, columns of C 2^62); test sums of a plane 2^62.6, an eighth of them
 // enters the transposed interpolation, whose sums stay below 2^62.5.  Sums of three products stay below 2^63 in
 // both words.  Each rounding is to nearest at 2^-53 to 2^-58 of the stage's bound, where floating point rounds
-// every operation, and the coefficients are formed from 106 bits: measured against extended precision the
-// operator's error is a third to a sixth of the FP64 column kernel's on random vectors and no larger on smooth ones
-// (tests/test_gpu_fixed_point.py).  One rounding to FP64 before the scatter.
+// every operation, and the coefficients are formed from 106 bits: measured against extended precision on six meshes the
+// operator's error is 0.10-0.37 of the FP64 column kernel's on random vectors, 0.15-0.62 on smooth ones and 0.19-0.49
+// under large pressures (tests/test_gpu_fixed_point.py asserts that it is no larger).  One rounding to FP64 before the
+// scatter.
 //
 // Measured (us, floating-point column kernel -> this kernel): 32^3 trilinear K 348 -> 97, A 264 -> 62, B^T 136 ->
 // 36, B 146 -> 32; 32^3 Cartesian K 401 -> 80, A 327 -> 52; 16^3 trilinear K 61 -> 19; 8^3 K 23 -> 11.  Bound by

@@ -198,20 +198,6 @@ __global__ void k_extract_inverse(const double *__restrict__ M, int nb, int n0, 
 
 namespace smf {
 
-__global__ void k_mdot_partial_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
-                                   const double *__restrict__ w, long long n, double *__restrict__ partial) {
-  pdl_enter();
-  __shared__ double sh[32];
-  const int nvec = ctl[0] + add;
-  for (int j = 0; j < nvec; ++j) {
-    const double *v = V + (long long)j * ldv;
-    double s = 0.0;
-    SMF_GRID_LOOP(i, n) s += v[i] * w[i];
-    s = block_reduce_sum<double>(s, sh);
-    if (threadIdx.x == 0) partial[(long long)j * gridDim.x + blockIdx.x] = s;
-  }
-}
-
 // The sums over a warp of eight values a lane, value (lane >> 2) in the result: each exchange also halves the values a
 // lane still holds, 9 additions instead of the 40 of eight separate reductions (a warp's FP64 addition occupies an
 // SM's FP64 unit for 19 clocks).
@@ -274,18 +260,6 @@ __global__ void k_mdot_final_cnt(const double *__restrict__ V, long long ldv, co
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) out[j] = s;
   }
-}
-
-__global__ void k_final_reduce_cnt(const double *__restrict__ partial, int nparts, const int *__restrict__ ctl, int add,
-                                   double *__restrict__ out) {
-  pdl_enter();
-  __shared__ double sh[32];
-  const int j = blockIdx.x;
-  if (j >= ctl[0] + add) return;  // uniform per block
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += partial[(long long)j * nparts + b];
-  s = block_reduce_sum<double>(s, sh);
-  if (threadIdx.x == 0) out[j] = s;
 }
 
 __global__ void k_maxpy_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,

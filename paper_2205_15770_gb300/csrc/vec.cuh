@@ -504,19 +504,11 @@ struct KrylovDev {
   unsigned *ticket = nullptr;  // finished blocks of k_mdot_final_cnt (returns to 0 after every launch)
   int m = 0;
 };
-// k_mdot_partial_cnt and k_final_reduce_cnt in one launch: every block writes its partial sums, the
-// last block to finish (a ticket counter, after a fence) sums them per vector in the same fixed
-// order as k_final_reduce_cnt and writes out[jj] for jj < ctl[0] + add (V == w, add == 1 - ctl[0]
-// gives ||w||^2 through ctl = null: then one vector, V = w).
+// out[jj] = V_jj . w for jj < ctl[0] + add: every block writes its partial sums, the last block to finish (a ticket
+// counter, after a fence) sums them per vector in a fixed order.
 __global__ void k_mdot_final_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
                                  const double *__restrict__ w, long long n, double *__restrict__ partial,
                                  unsigned *__restrict__ ticket, double *__restrict__ out);
-// partial[jj * gridDim.x + b] = block b's part of V_jj . w for jj < ctl[0] + add
-__global__ void k_mdot_partial_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
-                                   const double *__restrict__ w, long long n, double *__restrict__ partial);
-// out[jj] = sum_b partial[jj * nparts + b], one block per jj; blocks jj >= ctl[0] + add return
-__global__ void k_final_reduce_cnt(const double *__restrict__ partial, int nparts, const int *__restrict__ ctl, int add,
-                                   double *__restrict__ out);
 // w += sign * sum_{jj < ctl[0] + add} h[jj] V_jj
 __global__ void k_maxpy_cnt(const double *__restrict__ V, long long ldv, const int *__restrict__ ctl, int add,
                             const double *__restrict__ h, double *__restrict__ w, long long n, double sign);
