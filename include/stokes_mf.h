@@ -34,7 +34,8 @@
  *  - STOKES_NO_FUSE=1: unfused smoothing everywhere.  STOKES_NO_GRAPHS=1: no CUDA-graph capture.
  *  - STOKES_HOST_KRYLOV=1: the FGMRES iterations driven from the host (stokes_krylov_mode).
  *  - STOKES_BATCH_QUEUE=1: the batch's FP32 cycles in the persistent work-queue kernel.
- *  - STOKES_NO_EXPLICIT=1: the FP32 cycle of the small coarse levels by launches, not as an explicit matrix.
+ *  - STOKES_NO_EXPLICIT=1: the FP32 cycle of the small coarse levels by launches, not as an explicit matrix (FP32
+ *    entries, the sums with their rounding errors carried along in place of the coarse solve's FP64 sums).
  *  - STOKES_NO_SCHUR_MATRIX=1: S~ = B A^-1_hat B^T by its applications on every level, not as an explicit matrix
  *    (k = 2, kA = 1).
  *  - STOKES_NO_PLANE=1: FP32 launch shape 5 is the cell-component kernel, never the plane kernel (k = 2).
@@ -272,7 +273,12 @@ int stokes_solve_host(stokes_ctx *ctx, const double *b_host, double *x_host, dou
 /* Replace the per-cell viscosity of the finest level (HOST, n_cells positive doubles, x
  * fastest) and rebuild everything that depends on it (coarse viscosities = mean of the 2^d
  * children, diagonals, lambda_max estimates, coarse inverse).  Synchronises the stream; the
- * context pointer stays valid.  No counterpart in the paper (the paper's mu is constant). */
+ * context pointer stays valid.  The launch shapes and smoother forms that setup timed are kept.  The
+ * explicit S~ of the smoother (k = 2, kA = 1) is not built again: smoothing applies S~ block by block from
+ * the first change on, the same map at 1.2 to 1.4 times the time of a cycle with k_S = 1 (32^3 FP32 0.76 -> 0.92 ms), while
+ * the change itself takes 9 ms less at 16^3 cells, 19 at 32^3.  A caller that solves many times
+ * with one viscosity (more than about 20 FP32-cycle solves a change) is better served by a new context.
+ * No counterpart in the paper (the paper's mu is constant). */
 int stokes_set_viscosity(stokes_ctx *ctx, const double *mu_cell, void *stream);
 
 /* Adjoint viscosity gradient on the finest level: dJ_dmu[c] = - sum over velocity components of
@@ -399,7 +405,8 @@ int stokes_get_plane_form(const stokes_ctx *ctx, int level, int precision, int *
 
 /* 1 if smoothing on `level` / `precision` runs in the fused form (k_A = 1; the
  * Chebyshev-Jacobi and Uzawa vector updates of Sec. 3.3.1 evaluated inside the cell-kernel
- * gathers, 5 + 3 k_S launches per step, 5 + k_S with the explicit S~), 0 if in the unfused form (separate vector kernels).
+ * gathers, 5 + 3 k_S launches per step, 5 + k_S with the explicit S~), 0 if in the unfused form (separate
+ * vector kernels).
  * Setup times both forms per level and keeps the faster (STOKES_NO_AUTOTUNE=1: fused wherever
  * eligible; STOKES_NO_FUSE=1: never).  Level 0 (direct solve) reports 0.  HOST output. */
 int stokes_get_smoother_fusion(stokes_ctx *ctx, int level, int precision, int *fused);
