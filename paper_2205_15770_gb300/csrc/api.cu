@@ -444,7 +444,8 @@ struct Runner {
   std::vector<LevelRT<T>> &L;
   const Tab1D<T> *tab;
   int cols = 1;      // vectors handled by every launch, ld entries apart (setup; unfused forms)
-  long long ld = 0;
+  long long ld = 0;  // 0: the context's own vectors.  Otherwise a batch of columns, which may be a single one: the same
+                     // forms whatever its width, since the fused ones start from vectors that the unfused leave written
   explicit Runner(stokes_ctx *c) : C(c), s(c->s), L(levels<T>(c)), tab(tables<T>(c)) {}
   // several columns on their own work vectors
   Runner(stokes_ctx *c, std::vector<LevelRT<T>> &levels_, int cols_, long long ld_)
@@ -783,7 +784,7 @@ struct Runner {
   // step, residual) or written by k_fused_finish.
   bool fused_ok(int l) const { return fused_eligible(l) && L[l].fuse; }
   bool fused_eligible(int l) const {
-    return cols == 1 && C->fuse && !C->det && !hasC() && !C->sym && !L[l].rho && C->o.kA == 1 && C->o.kS >= 1 && C->o.kS <= 4 &&
+    return ld == 0 && C->fuse && !C->det && !hasC() && !C->sym && !L[l].rho && C->o.kA == 1 && C->o.kS >= 1 && C->o.kS <= 4 &&
            L[l].shape >= 0;
   }
   T *pairU(int l, int pr) { return pr == 0 ? L[l].tu : L[l].cx; }
@@ -1009,7 +1010,7 @@ struct Runner {
   // explicit matrix.
   void coarse_cycles(int l) {
     if constexpr (std::is_same<T, float>::value) {
-      if (l == C->le && cols == 1 && !rec()) {
+      if (l == C->le && ld == 0 && !rec()) {
         const int n = (int)(nu(l) + np(l));
         launch_kernel(k_explicit_apply, dim3((n + kExplicitWarps - 1) / kExplicitWarps), dim3(32 * kExplicitWarps), 0, s,
                       (const float *)C->Mx, n, C->ldm, (const float *)L[l].b, L[l].x);
