@@ -1489,14 +1489,19 @@ static int build_xfer(stokes_ctx *C, const LevelDesc<T> &F, const LevelDesc<T> &
 // Zero every smoother work vector of a level (accumulation targets must start at zero; the
 // unfused and fused smoothers leave different state vectors behind).
 template <typename T>
-static int zero_level_work(stokes_ctx *C, LevelRT<T> &R) {
+static int zero_level_work(LevelRT<T> &R, cudaStream_t s) {
   const long long nu = R.d.n_u, np = R.d.n_p;
   T *vel[] = {R.tu, R.ru, R.uhat, R.cx, R.cd, R.ct, R.r2, R.cx2, R.cd2, R.ct2, R.au};
-  for (T *p : vel) SMF_CUDA_OK(cudaMemsetAsync(p, 0, (size_t)nu * sizeof(T), C->s));
+  for (T *p : vel) SMF_CUDA_OK(cudaMemsetAsync(p, 0, (size_t)nu * sizeof(T), s));
   T *pre[] = {R.pt, R.rp, R.px, R.pd, R.ps, R.dp};
-  for (T *p : pre) SMF_CUDA_OK(cudaMemsetAsync(p, 0, (size_t)np * sizeof(T), C->s));
-  SMF_CUDA_OK(cudaMemsetAsync(R.kx, 0, (size_t)(nu + np) * sizeof(T), C->s));
+  for (T *p : pre) SMF_CUDA_OK(cudaMemsetAsync(p, 0, (size_t)np * sizeof(T), s));
+  SMF_CUDA_OK(cudaMemsetAsync(R.kx, 0, (size_t)(nu + np) * sizeof(T), s));
   return STOKES_OK;
+}
+
+template <typename T>
+static int zero_level_work(stokes_ctx *C, LevelRT<T> &R) {
+  return zero_level_work(R, C->s);
 }
 
 struct StreamGuard {
@@ -3063,6 +3068,25 @@ static bool batch_qbuild(stokes_batch *Bt) {
   return true;
 }
 
+// After a run of the queue (finished on Bt->s): its status, with the work vectors of the levels that smooth in the
+// fused form zero again for the members' own cycles, since the queue's unfused form leaves some written; of every level
+// after a run that gave up in the middle of its sums.
+static int queue_finish(stokes_batch *Bt) {
+  unsigned qerr = 0;
+  SMF_CUDA_OK(cudaMemcpyAsync(&qerr, Bt->qrun.state + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, Bt->s));
+  SMF_CUDA_OK(cudaStreamSynchronize(Bt->s));
+  for (auto *C : Bt->ctx)
+    for (int l = 1; l < C->nl; ++l)
+      if (qerr || Runner<float>(C).fused_ok(l))
+        if (const int st = zero_level_work(C->L32[l], Bt->s)) return st;
+  SMF_CUDA_OK(cudaStreamSynchronize(Bt->s));
+  if (qerr) {
+    set_error("batched work-queue kernel: a dependency wait exceeded its budget");
+    return STOKES_ETIMEOUT;
+  }
+  return STOKES_OK;
+}
+
 static int batch_solve(stokes_batch *Bt, const double *const *b, double *const *x, double rtol, int maxit, int *iters,
                        double *final_rel) {
   const int nm = (int)Bt->ctx.size();
@@ -3195,15 +3219,8 @@ static int batch_solve(stokes_batch *Bt, const double *const *b, double *const *
         st.it = hctl[1];
         st.need_start = true;
       }
-      if (Bt->kmode == 2) {
-        unsigned qerr = 0;
-        SMF_CUDA_OK(cudaMemcpyAsync(&qerr, Bt->qrun.state + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, Bt->s));
-        SMF_CUDA_OK(cudaStreamSynchronize(Bt->s));
-        if (qerr) {
-          set_error("batched work-queue kernel: a dependency wait exceeded its budget");
-          return STOKES_ETIMEOUT;
-        }
-      }
+      if (Bt->kmode == 2)
+        if (const int qs = queue_finish(Bt)) return qs;
       continue;
     }
     // (b) one Arnoldi step for every active mesh; the FP32 cycles of all meshes in one graph
@@ -4228,14 +4245,7 @@ int stokes_batch_vcycle(stokes_batch *Bt, const float *const *b, float *const *x
     const long long n = C->L32[top].d.n_u + C->L32[top].d.n_p;
     SMF_CUDA_OK(cudaMemcpyAsync(x[i], C->L32[top].x, n * sizeof(float), cudaMemcpyDeviceToDevice, Bt->s));
   }
-  unsigned qerr = 0;
-  SMF_CUDA_OK(cudaMemcpyAsync(&qerr, R.state + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, Bt->s));
-  SMF_CUDA_OK(cudaStreamSynchronize(Bt->s));
-  if (qerr) {
-    set_error("batched work-queue kernel: a dependency wait exceeded its budget");
-    return STOKES_ETIMEOUT;
-  }
-  return STOKES_OK;
+  return queue_finish(Bt);
 }
 int stokes_batch_set_wait_cycles(stokes_batch *Bt, unsigned int cycles) {
   if (!Bt) {
