@@ -3,6 +3,7 @@
 // FP64 flexible-GMRES outer loop.  Host code orchestrates; every vector operation runs
 // in the kernels of apply.cuh, vec.cuh, transfer.cuh and kernels_misc.cu.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <functional>
@@ -308,7 +309,14 @@ __global__ void k_fma_peak_x2(float *out, int iters, float seed) {
 
 using namespace smf;
 
+// A number no context has had: what was captured from a context holds while its number stays.
+static unsigned long long next_epoch() {
+  static std::atomic<unsigned long long> n{0};
+  return ++n;
+}
+
 struct stokes_ctx {
+  unsigned long long epoch = next_epoch();  // another after a change of viscosities or of a launch shape
   int dim = 0, k = 0, nl = 0;
   int device = -1;  // the CUDA device that was current at setup (every buffer lives there)
   stokes_opts o{};
@@ -2427,6 +2435,7 @@ static int det_check(stokes_ctx *C, cudaStream_t s) {
 
 // Destroys every captured graph of the context (cycles and the device Krylov loop).
 static void drop_graphs(stokes_ctx *C) {
+  C->epoch = next_epoch();
   for (int i = 0; i < 2; ++i) {
     if (C->g32[i].exec) cudaGraphExecDestroy(C->g32[i].exec);
     if (C->g64[i].exec) cudaGraphExecDestroy(C->g64[i].exec);
@@ -2737,9 +2746,26 @@ struct stokes_batch {
   PqRun qrun{};
   size_t qsmem = 0;
   unsigned qbudget = 0;
+  std::vector<unsigned long long> epochs;  // the members' when graph, kgraph and qmem were made
 };
 
 namespace smf {
+
+// Gives back what was captured or recorded from a member that has changed since (its vectors may have been freed).
+static int batch_refresh(stokes_batch *Bt) {
+  std::vector<unsigned long long> now;
+  for (auto *C : Bt->ctx) now.push_back(C->epoch);
+  if (now == Bt->epochs) return STOKES_OK;
+  SMF_CUDA_OK(cudaStreamSynchronize(Bt->s));
+  if (Bt->graph) cudaGraphExecDestroy(Bt->graph);
+  if (Bt->kgraph) cudaGraphExecDestroy(Bt->kgraph);
+  if (Bt->qmem) cudaFree(Bt->qmem);
+  Bt->graph = Bt->kgraph = nullptr;
+  Bt->qmem = nullptr;
+  Bt->kmode = -1;
+  Bt->epochs = now;
+  return STOKES_OK;
+}
 
 static int batch_capture(stokes_batch *Bt) {
   SMF_CUDA_OK(cudaStreamBeginCapture(Bt->s, cudaStreamCaptureModeThreadLocal));
@@ -3090,6 +3116,7 @@ static int queue_finish(stokes_batch *Bt) {
 static int batch_solve(stokes_batch *Bt, const double *const *b, double *const *x, double rtol, int maxit, int *iters,
                        double *final_rel) {
   const int nm = (int)Bt->ctx.size();
+  if (const int rs = batch_refresh(Bt)) return rs;
   if (Bt->kmode < 0) {
     const char *hk = getenv("STOKES_HOST_KRYLOV");
     const char *qe = getenv("STOKES_BATCH_QUEUE");
@@ -4219,6 +4246,7 @@ int stokes_batch_vcycle(stokes_batch *Bt, const float *const *b, float *const *x
       set_error("null vector in stokes_batch_vcycle");
       return STOKES_EINVAL;
     }
+  if (const int rs = batch_refresh(Bt)) return rs;
   if (!Bt->qmem && !batch_qrecord(Bt)) {
     set_error("stokes_batch_vcycle: the work-queue form does not serve this batch (every member 3D, k = 2, FP32 "
               "cycle, no stabilisation, symmetric gradient or rho term)");
