@@ -347,7 +347,8 @@ int stokes_setup_batch(int n_meshes, const stokes_mesh *meshes, const int *k, co
                        stokes_batch **out);
 
 /* The context of batch member `mesh` (owned by the batch; for sizes, right-hand sides, vmult):
- * *ctx is valid until stokes_destroy_batch and must not be destroyed by the caller.  STOKES_EINVAL
+ * *ctx is valid until stokes_destroy_batch and must not be destroyed by the caller; a change of its viscosities or
+ * launch shapes holds for the batched calls that follow, the first of which captures again.  STOKES_EINVAL
  * for an index out of range.  No counterpart in the paper (the batch layer). */
 int stokes_batch_context(stokes_batch *batch, int mesh, stokes_ctx **ctx);
 
